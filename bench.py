@@ -78,10 +78,10 @@ def thermalise_dynamical(lat, U, prm, ntraj, seed):
 
 PEAKS = os.path.join(ROOT, "MEASURED_PEAKS.json")
 
-# DRAM bytes per k_solve launch from the ncu capture summarised in
+# DRAM bytes per solver launch from the ncu capture summarised in
 # profiles/k_solve_16x16x16x32_f32.md, valid only for the solver source
 # that was captured (bench.py reports null once the source differs)
-SOLVER_SOURCES = ("lqcd_solver.cu", "lqcd_common.cuh", "lqcd_df.cuh")  # the sources k_solve is built from
+SOLVER_SOURCES = ("lqcd_split.cu", "lqcd_solve.cuh", "lqcd_common.cuh", "lqcd_df.cuh")  # the sources k_split is built from
 SOLVER_TRAFFIC = dict(src_sha256="aef4788cc714dda78760d271604c272fd83e3842839fc76a07edbe1288dfd3b3",
                       block_series=(303.767e6 + 154.127e6), block=(307.420e6 + 312.868e6),
                       glob=(392.167e6 + 425.938e6))
@@ -492,7 +492,7 @@ def run_ours(args):
                                           "%d series terms per block solve" % args.sap_terms)
                                     if args.global_solver == "sap-blocks" else "even-odd BiCGstab",
                    "dynamical_thermalisation": args.therm_fermion},
-        "roofline": {"bound": "hbm", "kernel": "persistent batched solver (k_solve)",
+        "roofline": {"bound": "hbm", "kernel": "persistent batched solver (k_split)",
                      "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": (achieved / peak) if achieved else None, "traffic": traffic,
                      "peak_kind": peak_kind, "launches": n_sol,

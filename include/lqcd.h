@@ -409,9 +409,9 @@ int lqcd_profile_times(lqcd_t h, int kernel_id, float* ms_out, int64_t cap, int6
 /* Launch schedules picked by measurement on this handle's lattice and
  * gauge field (the paper has no counterpart; its code ran on CPUs):
  * what & 1: threads per block of the hopping sweep (64 / 128 / 256), per
- * storage precision; what & 2: sites per thread of the persistent solver
- * (1 / 2, i.e. CTAs per system, or 0: every co-resident CTA with an equal
- * contiguous share of the sites), per precision, separately for the
+ * storage precision; what & 2: passes of the persistent solver's CTAs over
+ * their sites (1 / 2, i.e. CTAs per system, or 0: every co-resident CTA with
+ * an equal share of the sites), per precision, separately for the
  * batched slab solve and the global solve, each candidate timed on a
  * solve at `kappa` to 1e-10.  The choices stay with the handle; results
  * are the same up to rounding for every choice.  Synchronous.
@@ -421,8 +421,8 @@ int lqcd_profile_times(lqcd_t h, int kernel_id, float* ms_out, int64_t cap, int6
 int lqcd_autotune(lqcd_t h, int what, double kappa);
 int lqcd_tune_read(lqcd_t h, int* out);
 /* Sets the persistent solver's schedule of every precision and both solve
- * kinds to `spt` (1 or 2 sites per thread, 0 every co-resident CTA with an
- * equal share of the sites), as lqcd_autotune would pick it.  Results are
+ * kinds to `spt` (1 or 2 passes over the sites, 0 every co-resident CTA with
+ * an equal share of the sites), as lqcd_autotune would pick it.  Results are
  * the same up to rounding.  Errors: LQCD_ERR_ARG (spt outside 0..2). */
 int lqcd_set_solver_schedule(lqcd_t h, int spt);
 /* enable = 1: single-precision geometric-series slab solves (the sub-slab

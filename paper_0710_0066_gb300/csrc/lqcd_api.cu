@@ -977,7 +977,7 @@ int lqcd_create(lqcd_t* out, const int L[4], int l0, int bc_t, void* stream)
     const size_t Vh = g.Vh;
     LQ_CUDA(h, cudaMalloc(&h->U64, sizeof(double2) * 72 * Vh));
     LQ_CUDA(h, cudaMalloc(&h->U64_save, sizeof(double2) * 72 * Vh));
-    LQ_CUDA(h, cudaMalloc(&h->U32, sizeof(float4) * 24 * Vh));
+    LQ_CUDA(h, cudaMalloc(&h->U32, sizeof(float4) * 8 * link32_block(g.Vh)));
     LQ_CUDA(h, cudaMalloc(&h->U16, sizeof(uint2) * 48 * Vh));  // fp16, then bf16
     h->f64.assign(NFIELD, nullptr);
     for (int k = 0; k < NFIELD; ++k) LQ_CUDA(h, cudaMalloc(&h->f64[k], sizeof(double2) * 24 * Vh));

@@ -8,7 +8,9 @@
 //                  + [parity][Vh] float scale (max |component| of the site)
 //   bf16 spinor    [parity][3][Vh]            uint4   (four complex each, no scale)
 //   double gauge   [mu][parity][9][Vh]        double2 (full 3x3)
-//   single gauge   [mu][parity][3][Vh]        float4  (rows 0 and 1)
+//   single gauge   [mu][parity][Vh/32][3][32] float4  (rows 0 and 1): tiles of 32
+//                  sites (Vh rounded up), so that one address and constant
+//                  offsets reach the three words of a link
 //   half gauge     [mu][parity][3][Vh]        uint2   (rows 0 and 1)
 //   bf16 gauge     the same, following the half gauge in one allocation
 // Row 2 of a compressed link is rebuilt as conj(row0 x row1) (SU(3)).
@@ -541,13 +543,18 @@ __device__ __forceinline__ void load_link<PRECDS>(const GaugeF& g, int mu, int p
 {
     load_link<PRECDF>(g, mu, par, i, u);
 }
+// words of one (mu, parity) block of the single-precision links, and the
+// place of word 0 of link i in it (word k: 32 k further)
+LQ_HD size_t link32_block(int Vh) { return (size_t)((Vh + 31) & ~31) * 3; }
+LQ_HD int link32_at(int i) { return i + (i >> 5) * 64; }
+
 template <>
 __device__ __forceinline__ void load_link<PREC32>(const GaugeF& g, int mu, int par, int i, Su3<float>& u)
 {
-    const float4* p = (const float4*)g.v + (size_t)(mu * 2 + par) * 3 * g.Vh;
+    const float4* p = (const float4*)g.v + (size_t)(mu * 2 + par) * link32_block(g.Vh) + link32_at(i);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        float4 d = __ldg(p + (size_t)k * g.Vh + i);
+        float4 d = __ldg(p + 32 * k);
         u.m[(2 * k) / 3][(2 * k) % 3] = mk(d.x, d.y);
         u.m[(2 * k + 1) / 3][(2 * k + 1) % 3] = mk(d.z, d.w);
     }
@@ -575,7 +582,7 @@ __device__ __forceinline__ void store_low_link_word(float4* U32, uint2* U16, int
                                                     double xi, double yr, double yi)
 {
     const size_t o = (size_t)mp * 3 * Vh + (size_t)k * Vh + i;
-    U32[o] = make_float4((float)xr, (float)xi, (float)yr, (float)yi);
+    U32[(size_t)mp * link32_block(Vh) + link32_at(i) + 32 * k] = make_float4((float)xr, (float)xi, (float)yr, (float)yi);
     __half2 hx = __floats2half2_rn((float)xr, (float)xi);
     __half2 hy = __floats2half2_rn((float)yr, (float)yi);
     U16[o] = make_uint2(*reinterpret_cast<unsigned*>(&hx), *reinterpret_cast<unsigned*>(&hy));
@@ -806,6 +813,91 @@ __device__ __forceinline__ void hop_site_df(const Geo& g, int mode, int dag, int
     }
 }
 
+// One colour r of the hopping term at (pout, i), all four spins, for the
+// double sweeps of the persistent solver: three work items per site with 16
+// instead of 48 accumulator registers (double-float), at the price of
+// projecting every neighbour once per colour (17 % more arithmetic; its
+// loads repeat out of L1).
+LQ_HD double as_double(double v) { return v; }
+LQ_HD double as_double(df v) { return df_to_double(v); }
+
+template <int P, bool RO>
+__device__ __forceinline__ cx<typename Real<P>::T> load_comp(const SpinorF& f, int c, int j)
+{
+    if constexpr (P == PREC64) {
+        const double2 d = ldv<double2, RO>((const double2*)f.v + (size_t)c * f.N + j);
+        return mk(d.x, d.y);
+    } else {
+        return df_in<P, RO>(f, c, j);
+    }
+}
+template <int P>
+__device__ __forceinline__ void store_comp(const SpinorF& f, int c, int j, cx<typename Real<P>::T> v)
+{
+    if constexpr (P == PREC64)
+        ((double2*)f.v)[(size_t)c * f.N + j] = make_double2(v.re, v.im);
+    else
+        ((float4*)f.v)[(size_t)c * f.N + j] = make_float4(v.re.hi, v.im.hi, v.re.lo, v.im.lo);
+}
+
+template <int P, bool RO>
+__device__ __forceinline__ void hop_colour(const Geo& g, int mode, int dag, int pout, int i, int r, const SpinorF& in,
+                                           const GaugeF& U, cx<typename Real<P>::T> acc[4])
+{
+    typedef typename Real<P>::T T;
+#pragma unroll
+    for (int s = 0; s < 4; ++s) acc[s] = mk(T(0), T(0));
+    int x[4];
+    eo_coords(g, pout, i, x);
+    const int lex = lex_of(g, x);
+    int stride = 1;
+#pragma unroll 1
+    for (int mu = 3; mu >= 0; --mu) {
+        const int xm = mu == 3 ? x[3] : mu == 2 ? x[2] : mu == 1 ? x[1] : x[0];
+        const int Lm = mu == 3 ? g.L[3] : mu == 2 ? g.L[2] : mu == 1 ? g.L[1] : g.L[0];
+#pragma unroll
+        for (int fw = 1; fw >= 0; --fw) {
+            int nl = fw ? lex + stride : lex - stride;
+            const bool wrap = fw ? (xm == Lm - 1) : (xm == 0);
+            if (wrap) nl += fw ? -Lm * stride : Lm * stride;
+            bool use = true;
+            if (mu == 0) use = t_hop_kept(g, mode, fw ? x[0] + 1 : x[0]);
+            else if (mode == MODE_CROSS || mode == MODE_CROSS2) use = false;
+            if (!use) continue;
+            const int j = nl >> 1;
+            const int sg = fw ? (dag ? +1 : -1) : (dag ? -1 : +1);
+            const double2* up = (const double2*)U.v + (size_t)(mu * 2 + (fw ? pout : 1 - pout)) * 9 * U.Vh + (fw ? i : j);
+            cx<T> w0 = mk(T(0), T(0)), w1 = w0;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                cx<T> h0, h1;
+                project1(mu, sg, load_comp<P, RO>(in, c, j), load_comp<P, RO>(in, 3 + c, j), load_comp<P, RO>(in, 6 + c, j),
+                         load_comp<P, RO>(in, 9 + c, j), h0, h1);
+                const double2 d = __ldg(up + (size_t)(fw ? 3 * r + c : 3 * c + r) * U.Vh);
+                const cx<T> u = mk(T(d.x), fw ? T(d.y) : T(-d.y));
+                w0 = c ? w0 + u * h0 : u * h0;
+                w1 = c ? w1 + u * h1 : u * h1;
+            }
+            if (mu == 0 && wrap && g.bc_t < 0) {
+                w0 = -w0;
+                w1 = -w1;
+            }
+            acc[0] = acc[0] + w0;
+            acc[1] = acc[1] + w1;
+            cx<T> l0, l1;
+            switch (mu) {
+                case 0: l0 = -w0; l1 = -w1; break;
+                case 1: l0 = mul_i(w1); l1 = mul_i(w0); break;
+                case 2: l0 = w1; l1 = -w0; break;
+                default: l0 = mul_i(w0); l1 = mul_mi(w1); break;
+            }
+            if (sg < 0) { acc[2] = acc[2] - l0; acc[3] = acc[3] - l1; }
+            else        { acc[2] = acc[2] + l0; acc[3] = acc[3] + l1; }
+        }
+        stride *= Lm;
+    }
+}
+
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
@@ -844,7 +936,7 @@ struct lqcd_ctx {
     bool have_gauge = false;
     // internal gauge copies
     double2* U64 = nullptr;  // [4][2][9][Vh]
-    float4* U32 = nullptr;   // [4][2][3][Vh]
+    float4* U32 = nullptr;   // [4][2][Vh/32][3][32]
     uint2* U16 = nullptr;    // [4][2][3][Vh] fp16, then [4][2][3][Vh] bf16
     double2* U64_save = nullptr;
     // double full-lattice spinor scratch fields [2][12][Vh]

@@ -8,6 +8,9 @@
 //   inner loop (double, single or half storage, FP32 arithmetic):
 //     BiCGstab on A e = r / |r| to a relative residual inner_tol;
 //   x += |r| e.
+// Double and single precision without Schwarz preconditioner run in
+// lqcd_split.cu; k_solve here runs the half formats and every
+// Schwarz-preconditioned solve, k_series_cl the opt-in cluster form.
 // Each system is handled by its own group of CTAs (cps CTAs per system).
 // Reductions are per system, in double, in a fixed order (warp shuffles,
 // then the group's per-CTA partials summed in CTA order), so every CTA of a
@@ -24,7 +27,7 @@
 
 #include <cooperative_groups.h>
 
-#include "lqcd_common.cuh"
+#include "lqcd_solve.cuh"
 
 namespace {
 
@@ -41,72 +44,6 @@ constexpr int SOLVE_UNR = LQCD_SOLVE_UNR;
 // (measured at 16^3 x 32: rolled BiCGstab 11 % faster, rolled series 10 %
 // slower)
 constexpr int SERIES_UNR = 4;
-constexpr int NSYS_MAX = 64;
-constexpr int NQ = 3;
-constexpr int NACC = 5;  // iteration sums kept beside the sticky status
-
-// per-system state codes in the flag arrays
-enum { F_ACTIVE = 0, F_DONE = 1, F_NAN = 2, F_MAXIT = 3 };
-
-struct SolveArgs {
-    Geo g;
-    int mode;  // MODE_INTRA: slabs, MODE_ALL: whole lattice
-    double k2;
-    double diag;  // the system is diag - k2 H_eo H_oe (1, or 1 + rho for W3,eo)
-    int method;   // SOLVER_BICGSTAB or SOLVER_SERIES (inner iteration)
-    int guess;    // 1: x holds an initial guess on entry, 0: start from x = 0
-    int nsys, cps;
-    int chunk;  // sites of one system handled by one CTA (the last CTA may get fewer)
-    int slab0, slabstep;
-    int nsite;
-    GaugeF U64, UP;
-    SpinorF b, x, r64;  // double, parity 0
-    SpinorF t64;        // parity 1: double (double solve) or df pairs (mixed)
-    SpinorF r, rh, p, v, s, t;  // inner precision, parity 0
-    SpinorF tmp;        // inner precision, parity 1
-    SpinorF e;          // inner solution (single; double for the double solver)
-    double tol, inner_tol;
-    int max_iter, max_outer, max_inner;
-    double* part;       // [NQ][grid]
-    unsigned* bar;      // one barrier counter per system, BAR_STRIDE apart
-    int* status;
-    int* sticky;        // first failure of any solve since the host last read it
-    unsigned long long* acc;  // [5] inner iterations, BiCGstab iterations x sites,
-                              // outer cycles x sites, series iterations x sites,
-                              // Schwarz-preconditioned iterations x sites
-    int* iters;         // [nsys]
-    double* resid;      // [nsys]
-    int* outer_out;
-    long long spin_limit;  // clock64 cycles of one barrier wait before LQCD_ERR_TIMEOUT
-    // Schwarz-preconditioned inner solve of the whole lattice (SOLVER_SAP):
-    // full-lattice vectors in the inner precision, [0] the even, [1] the odd
-    // parity block; fy (the inner solution) in the precision of e, whose
-    // even block it is
-    double kappa;
-    int nsap;  // geometric-series terms of every block solve of the preconditioner
-    // SOLVER_SAPB: 4-D Schwarz blocks of extents bk[mu] (2 or 4, lbk = log2),
-    // nbk[mu] = L[mu] / bk[mu] blocks per direction, nblk in all, bvh sites
-    // of one parity in a block
-    int bk[4], lbk[4], nbk[4], nblk, bvh;
-    SpinorF fr[2], frh[2], fp[2], fv[2], fs[2], ft[2], fzp[2], fzs[2], fw1[2], fw2[2], fy[2];
-};
-
-struct SysSt {  // the CTA's own system
-    double bn2, rn2, rr, itol2;
-    double2 rho, alpha, omega, beta;
-    int active, idone, it, itc, flag;
-};
-
-// barrier counters of different systems sit on different 128-byte lines
-constexpr int BAR_STRIDE = 32;
-
-__device__ __forceinline__ unsigned ld_acquire(const unsigned* p)
-{
-    unsigned v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
 // barrier over the cps CTAs of one system (the systems are independent and
 // never wait for one another); bounded: gives up after A.spin_limit cycles
 __device__ bool sys_sync(const SolveArgs& A, int sys, unsigned& epoch)
@@ -224,60 +161,12 @@ __device__ __forceinline__ bool finite2(double2 a) { return isfinite(a.x) && isf
 #define FOR_SITES                                                                                   \
     for (int j_ = cin * A.chunk + (int)threadIdx.x, je_ = min(A.nsite, (cin + 1) * A.chunk); j_ < je_; \
          j_ += SBS)
-// element-wise phases of the single-precision inner solver run over 16-byte
-// words (one float4 = two complex components) instead of whole sites: six
-// times the parallelism and few live registers per thread
+// the single-precision solution update runs over 16-byte words (one float4 =
+// two complex components) instead of whole sites
 #define FOR_WORDS for (int f_ = cin * SBS + (int)threadIdx.x; f_ < 6 * A.nsite; f_ += A.cps * SBS)
-#define WORD_ADDR const size_t a = (size_t)(f_ / A.nsite) * A.g.Vh + base + (f_ % A.nsite)
 #define W4(f) ((float4*)(f).v)
 #define SYNC_OR_RETURN \
     if (!sys_sync(A, sys, epoch)) return
-
-// y + a x for the two complex numbers of a word
-__device__ __forceinline__ float4 caxpy2(float2 a, float4 x, float4 y)
-{
-    return make_float4(y.x + a.x * x.x - a.y * x.y, y.y + a.x * x.y + a.y * x.x, y.z + a.x * x.z - a.y * x.w,
-                       y.w + a.x * x.w + a.y * x.z);
-}
-// word-parallel dot products: each thread sums its few words in FP32 and
-// hands the sum to the FP64 reduction once (GB300 issues FP64 at a small
-// fraction of the FP32 rate; the single-precision inner solver's scalars
-// need no more than FP32 accuracy per thread)
-__device__ __forceinline__ void cdot2(float4 a, float4 b, float& re, float& im)
-{
-    re += a.x * b.x + a.y * b.y + a.z * b.z + a.w * b.w;
-    im += a.x * b.y - a.y * b.x + a.z * b.w - a.w * b.z;
-}
-__device__ __forceinline__ float nrm2w(float4 a) { return a.x * a.x + a.y * a.y + a.z * a.z + a.w * a.w; }
-
-// single-precision spinor at site j of the combination y + a x of two
-// inner vectors (word by word, as the element-wise phases form it), and of
-// y + b (z + a x) of three
-__device__ __forceinline__ void load_axpy32(const SpinorF& x, const SpinorF& y, float2 a, int j, Spinor<float>& s)
-{
-    const float4* xp = (const float4*)x.v;
-    const float4* yp = (const float4*)y.v;
-#pragma unroll
-    for (int k = 0; k < 6; ++k) {
-        const float4 w = caxpy2(a, xp[(size_t)k * x.N + j], yp[(size_t)k * y.N + j]);
-        s.c[(2 * k) / 3][(2 * k) % 3] = mk(w.x, w.y);
-        s.c[(2 * k + 1) / 3][(2 * k + 1) % 3] = mk(w.z, w.w);
-    }
-}
-__device__ __forceinline__ void load_axpypz32(const SpinorF& x, const SpinorF& z, const SpinorF& y, float2 a, float2 b,
-                                              int j, Spinor<float>& s)
-{
-    const float4* xp = (const float4*)x.v;
-    const float4* zp = (const float4*)z.v;
-    const float4* yp = (const float4*)y.v;
-#pragma unroll
-    for (int k = 0; k < 6; ++k) {
-        const size_t o = (size_t)k * x.N + j;
-        const float4 w = caxpy2(b, caxpy2(a, xp[o], zp[o]), yp[o]);
-        s.c[(2 * k) / 3][(2 * k) % 3] = mk(w.x, w.y);
-        s.c[(2 * k + 1) / 3][(2 * k + 1) % 3] = mk(w.z, w.w);
-    }
-}
 
 template <class T>
 __device__ __forceinline__ void sp_axpy(Spinor<T>& y, T a, const Spinor<T>& x)  // y <- x + a y
@@ -931,7 +820,7 @@ __global__ void __launch_bounds__(SBS, P == PREC64 ? 1 : 2) k_solve(SolveArgs A)
     // t64 = H_oe x between the two residual sweeps: kept as df pairs in the
     // mixed case (no conversion to double and back)
     constexpr int PT = (P == PREC64) ? PREC64 : PRECDS;
-    constexpr bool WORDS = (P == PREC32);
+    constexpr bool WORDS = (P == PREC32);  // the solution update of the single-precision Schwarz solve
     const int cta = blockIdx.x, tid = threadIdx.x;
     const int sys = cta / A.cps, cin = cta - sys * A.cps;
     const bool leader = (cin == 0 && tid == 0);  // writes the system's results
@@ -1035,25 +924,7 @@ __global__ void __launch_bounds__(SBS, P == PREC64 ? 1 : 2) k_solve(SolveArgs A)
         // ---- inner start: r = rh = p = r64 / |r64|, e = 0
         {
             double q = 0.0;
-            if (S.active && WORDS) {
-                const double sc = 1.0 / sqrt(S.rn2);
-                const double2* r6 = (const double2*)A.r64.v;
-                float qf = 0.f;
-                FOR_WORDS
-                {
-                    const int k = f_ / A.nsite, i = base + (f_ % A.nsite);
-                    const size_t a = (size_t)k * A.g.Vh + i;
-                    const double2 d0 = r6[(size_t)(2 * k) * A.g.Vh + i], d1 = r6[(size_t)(2 * k + 1) * A.g.Vh + i];
-                    const float4 w = make_float4((float)(sc * d0.x), (float)(sc * d0.y), (float)(sc * d1.x),
-                                                 (float)(sc * d1.y));
-                    W4(A.r)[a] = w;
-                    W4(A.rh)[a] = w;
-                    W4(A.p)[a] = w;
-                    W4(A.e)[a] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    qf += nrm2w(w);
-                }
-                q = qf;
-            } else if (S.active) {
+            if (S.active) {
                 const double sc = 1.0 / sqrt(S.rn2);
                 FOR_SITES
                 {
@@ -1173,167 +1044,6 @@ __global__ void __launch_bounds__(SBS, P == PREC64 ? 1 : 2) k_solve(SolveArgs A)
                 }
             SYNC_OR_RETURN;
         } else {
-        if constexpr (P == PREC32) {
-            // ---- BiCGstab with the vector updates folded into the hopping
-            // phases: s = r - alpha v is formed where H_oe s reads it (at the
-            // neighbours) and where the next phase keeps it; the update
-            // p = r + beta (p - omega v) waits for the next iteration, whose
-            // H_oe p forms it at the neighbours and whose second phase keeps
-            // it.  Five barriers per iteration (seven unfolded); the same
-            // word-wise single-precision operations as the unfolded form.
-            bool pend = false;  // p = r + beta (p - omega v) not yet formed
-            const T k2 = (T)A.k2, dg = (T)A.diag;
-            for (;;) {
-                if (S.idone) break;
-                const float2 pbe = make_float2((float)S.beta.x, (float)S.beta.y);
-                const float2 pmom = make_float2(-(float)S.omega.x, -(float)S.omega.y);
-                // tmp = H_oe p'
-                if (pend) {
-                    FOR_SITES
-                    {
-                        const int i = base + j_;
-                        Spinor<T> a;
-                        hop_site_ld<P, SOLVE_UNR>(A.g, A.mode, 0, 1, i,
-                                       [&](int j, Spinor<T>& sp) { load_axpypz32(A.v, A.p, A.r, pmom, pbe, j, sp); },
-                                       A.UP, a);
-                        store_spinor<P>(A.tmp, i, a);
-                    }
-                } else {
-                    FOR_SITES
-                    {
-                        const int i = base + j_;
-                        Spinor<T> a;
-                        hop_site<P, false, SOLVE_UNR>(A.g, A.mode, 0, 1, i, A.p, A.UP, a);
-                        store_spinor<P>(A.tmp, i, a);
-                    }
-                }
-                SYNC_OR_RETURN;
-                // p = p' ; v = dg p - k2 H_eo tmp ; <rh, v>
-                {
-                    double qr = 0.0, qi = 0.0;
-                    FOR_SITES
-                    {
-                        const int i = base + j_;
-                        Spinor<T> a, pp, rh;
-                        hop_site<P, false, SOLVE_UNR>(A.g, A.mode, 0, 0, i, A.tmp, A.UP, a);
-                        if (pend) {
-                            load_axpypz32(A.v, A.p, A.r, pmom, pbe, i, pp);
-                            store_spinor<P>(A.p, i, pp);
-                        } else {
-                            load_spinor<P, false>(A.p, i, pp);
-                        }
-#pragma unroll
-                        for (int s = 0; s < 4; ++s)
-#pragma unroll
-                            for (int c = 0; c < 3; ++c) a.c[s][c] = dg * pp.c[s][c] - k2 * a.c[s][c];
-                        store_spinor<P>(A.v, i, a);
-                        load_spinor<P, false>(A.rh, i, rh);
-                        cdot_acc(rh, a, qr, qi);
-                    }
-                    reduce_put(A, qr, qi, 0.0, 2, rb);
-                    SYNC_OR_RETURN;
-                    gather_own(A, sys, 2, red, rb);
-                    if (tid == 0) {
-                        const double2 d = make_double2(red[0], red[1]);
-                        const double2 al = cdiv(S.rho, d);
-                        if (!finite2(al) || (d.x == 0.0 && d.y == 0.0)) {
-                            S.idone = 1;
-                            S.alpha = make_double2(0.0, 0.0);
-                        } else {
-                            S.alpha = al;
-                        }
-                    }
-                    __syncthreads();
-                }
-                pend = false;
-                if (S.idone) break;
-                const float2 mal = make_float2(-(float)S.alpha.x, -(float)S.alpha.y);
-                // tmp = H_oe s, s = r - alpha v formed at the neighbours
-                FOR_SITES
-                {
-                    const int i = base + j_;
-                    Spinor<T> a;
-                    hop_site_ld<P, SOLVE_UNR>(A.g, A.mode, 0, 1, i,
-                                   [&](int j, Spinor<T>& sp) { load_axpy32(A.v, A.r, mal, j, sp); }, A.UP, a);
-                    store_spinor<P>(A.tmp, i, a);
-                }
-                SYNC_OR_RETURN;
-                // s = r - alpha v (kept) ; t = dg s - k2 H_eo tmp ; <t, s>, <t, t>
-                {
-                    double qr = 0.0, qi = 0.0, qt = 0.0;
-                    FOR_SITES
-                    {
-                        const int i = base + j_;
-                        Spinor<T> a, ss;
-                        hop_site<P, false, SOLVE_UNR>(A.g, A.mode, 0, 0, i, A.tmp, A.UP, a);
-                        load_axpy32(A.v, A.r, mal, i, ss);
-                        store_spinor<P>(A.s, i, ss);
-#pragma unroll
-                        for (int s = 0; s < 4; ++s)
-#pragma unroll
-                            for (int c = 0; c < 3; ++c) a.c[s][c] = dg * ss.c[s][c] - k2 * a.c[s][c];
-                        store_spinor<P>(A.t, i, a);
-                        cdot_acc(a, ss, qr, qi);
-                        qt += nrm_acc(a);
-                    }
-                    reduce_put(A, qr, qi, qt, 3, rb);
-                    SYNC_OR_RETURN;
-                    gather_own(A, sys, 3, red, rb);
-                    if (tid == 0) {
-                        const double tt = red[2];
-                        const double2 om = make_double2(red[0] / tt, red[1] / tt);
-                        if (!(tt > 0.0) || !finite2(om)) {
-                            S.omega = make_double2(0.0, 0.0);
-                            S.idone = 2;  // keep alpha p, stop afterwards
-                        } else {
-                            S.omega = om;
-                        }
-                    }
-                    __syncthreads();
-                }
-                // e += alpha p + omega s ; r = s - omega t ; <rh, r>, |r|^2
-                {
-                    double qr = 0.0, qi = 0.0, qn = 0.0;
-                    const float2 al = make_float2((float)S.alpha.x, (float)S.alpha.y);
-                    const float2 om = make_float2((float)S.omega.x, (float)S.omega.y);
-                    const float2 mom = make_float2(-om.x, -om.y);
-                    float fr = 0.f, fi = 0.f, fn = 0.f;
-                    FOR_WORDS
-                    {
-                        WORD_ADDR;
-                        const float4 ss = W4(A.s)[a];
-                        W4(A.e)[a] = caxpy2(om, ss, caxpy2(al, W4(A.p)[a], W4(A.e)[a]));
-                        const float4 rr = caxpy2(mom, W4(A.t)[a], ss);
-                        W4(A.r)[a] = rr;
-                        cdot2(W4(A.rh)[a], rr, fr, fi);
-                        fn += nrm2w(rr);
-                    }
-                    qr = fr;
-                    qi = fi;
-                    qn = fn;
-                    reduce_put(A, qr, qi, qn, 3, rb);
-                    SYNC_OR_RETURN;
-                    gather_own(A, sys, 3, red, rb);
-                    if (tid == 0) {
-                        S.it += 1;
-                        S.itc += 1;
-                        const double2 rn = make_double2(red[0], red[1]);
-                        S.rr = red[2];
-                        if (S.idone == 2 || S.itc >= A.max_inner || S.it >= A.max_iter || !(S.rr > S.itol2) ||
-                            !finite2(rn) || S.rr > 1e8) {
-                            S.idone = 1;
-                        } else {
-                            S.beta = cmul(cdiv(rn, S.rho), cdiv(S.alpha, S.omega));
-                            if (!finite2(S.beta)) S.idone = 1;
-                            S.rho = rn;
-                        }
-                    }
-                    if (tid == 0 && S.idone) S.idone = 1;
-                    __syncthreads();
-                }
-                pend = !S.idone;
-            }
-        } else
         // ---- BiCGstab: seven barriers per iteration
         for (;;) {
             if (S.idone) break;
@@ -1385,14 +1095,7 @@ __global__ void __launch_bounds__(SBS, P == PREC64 ? 1 : 2) k_solve(SolveArgs A)
             }
             const bool act2 = act && !S.idone;
             // s = r - alpha v
-            if (act2 && WORDS) {
-                const float2 al = make_float2(-(float)S.alpha.x, -(float)S.alpha.y);
-                FOR_WORDS
-                {
-                    WORD_ADDR;
-                    W4(A.s)[a] = caxpy2(al, W4(A.v)[a], W4(A.r)[a]);
-                }
-            } else if (act2) {
+            if (act2) {
                 const cx<T> al = mk((T)S.alpha.x, (T)S.alpha.y);
                 FOR_SITES
                 {
@@ -1456,25 +1159,7 @@ __global__ void __launch_bounds__(SBS, P == PREC64 ? 1 : 2) k_solve(SolveArgs A)
             // e += alpha p + omega s ; r = s - omega t ; <rh, r>, |r|^2
             {
                 double qr = 0.0, qi = 0.0, qn = 0.0;
-                if (act2 && WORDS) {
-                    const float2 al = make_float2((float)S.alpha.x, (float)S.alpha.y);
-                    const float2 om = make_float2((float)S.omega.x, (float)S.omega.y);
-                    const float2 mom = make_float2(-om.x, -om.y);
-                    float fr = 0.f, fi = 0.f, fn = 0.f;
-                    FOR_WORDS
-                    {
-                        WORD_ADDR;
-                        const float4 ss = W4(A.s)[a];
-                        W4(A.e)[a] = caxpy2(om, ss, caxpy2(al, W4(A.p)[a], W4(A.e)[a]));
-                        const float4 rr = caxpy2(mom, W4(A.t)[a], ss);
-                        W4(A.r)[a] = rr;
-                        cdot2(W4(A.rh)[a], rr, fr, fi);
-                        fn += nrm2w(rr);
-                    }
-                    qr = fr;
-                    qi = fi;
-                    qn = fn;
-                } else if (act2) {
+                if (act2) {
                     const cx<T> al = mk((T)S.alpha.x, (T)S.alpha.y);
                     const cx<T> om = mk((T)S.omega.x, (T)S.omega.y);
                     FOR_SITES
@@ -1527,15 +1212,7 @@ __global__ void __launch_bounds__(SBS, P == PREC64 ? 1 : 2) k_solve(SolveArgs A)
                 __syncthreads();
             }
             // p = r + beta (p - omega v)
-            if (act2 && !S.idone && WORDS) {
-                const float2 be = make_float2((float)S.beta.x, (float)S.beta.y);
-                const float2 mom = make_float2(-(float)S.omega.x, -(float)S.omega.y);
-                FOR_WORDS
-                {
-                    WORD_ADDR;
-                    W4(A.p)[a] = caxpy2(be, caxpy2(mom, W4(A.v)[a], W4(A.p)[a]), W4(A.r)[a]);
-                }
-            } else if (act2 && !S.idone) {
+            if (act2 && !S.idone) {
                 const cx<T> be = mk((T)S.beta.x, (T)S.beta.y);
                 const cx<T> om = mk((T)S.omega.x, (T)S.omega.y);
                 FOR_SITES
@@ -1646,7 +1323,6 @@ __global__ void __launch_bounds__(SBS, P == PREC64 ? 1 : 2) k_solve(SolveArgs A)
 
 #undef FOR_SITES
 #undef FOR_WORDS
-#undef WORD_ADDR
 #undef W4
 #undef SYNC_OR_RETURN
 
@@ -2093,7 +1769,8 @@ struct Work {
     int* outer = nullptr;
     int* h_status = nullptr;  // pinned mirror: status, outer, iters[NSYS_MAX]
     double* h_resid = nullptr;
-    int gmax[NPREC] = {0, 0, 0, 0};  // co-resident CTAs per precision
+    int gmax[NPREC] = {0, 0, 0, 0};  // co-resident CTAs of k_solve per precision
+    int split_occ[SPLIT_NVAR][2];    // CTAs per SM of the k_split variants
     int cl_ok = 0;                   // the device runs k_series_cl's clusters
     // the Schwarz-preconditioned global solve: 11 full-lattice vectors, each
     // sized for a double full field (allocated on first use)
@@ -2134,14 +1811,13 @@ int solver_init(lqcd_ctx* h)
     Work* w = new Work();
     h->work = w;
     const int Vh = h->g.Vh;
-    for (int k = 0; k < 8; ++k) LQ_CUDA(h, cudaMalloc(&w->vec[k], sizeof(double2) * 12 * (size_t)Vh));
+    // the tiled vectors of lqcd_split.cu end on a full tile of 32 sites
+    for (int k = 0; k < 8; ++k) LQ_CUDA(h, cudaMalloc(&w->vec[k], sizeof(double2) * 12 * (size_t)((Vh + 31) & ~31)));
     LQ_CUDA(h, cudaMalloc(&w->r64, sizeof(double2) * 12 * (size_t)Vh));
     LQ_CUDA(h, cudaMalloc(&w->t64, sizeof(double2) * 12 * (size_t)Vh));
     // co-resident CTAs of a cooperative launch: the smaller occupancy of the
-    // two variants of each precision
-    int occ[NPREC], occs[NPREC];
-    LQ_CUDA(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[0], k_solve<PREC64, false>, SBS, 0));
-    LQ_CUDA(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[1], k_solve<PREC32, false>, SBS, 0));
+    // variants of each precision (single and double: the Schwarz one only)
+    int occ[NPREC] = {1 << 20, 1 << 20, 0, 0}, occs[NPREC];
     LQ_CUDA(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[2], k_solve<PREC16, false>, SBS, 0));
     LQ_CUDA(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[3], k_solve<PRECBF, false>, SBS, 0));
     // the Schwarz variants run with the 4-D block preconditioner's dynamic
@@ -2183,7 +1859,9 @@ int solver_init(lqcd_ctx* h)
         w->gmax[k] = std::max(1, std::min(occ[k], occs[k])) * h->num_sms;
         gm = std::max(gm, w->gmax[k]);
     }
-    LQ_CUDA(h, cudaMalloc(&w->part, sizeof(double) * 2 * NQ * (size_t)gm));
+    int gsplit = 0;
+    LQ_CUDA(h, split_init(h->num_sms, w->split_occ, &gsplit));
+    LQ_CUDA(h, cudaMalloc(&w->part, sizeof(double) * 2 * std::max(NQ * (size_t)gm, SPLIT_NQ * (size_t)gsplit)));
     LQ_CUDA(h, cudaMalloc(&w->bar, sizeof(unsigned) * BAR_STRIDE * NSYS_MAX));
     LQ_CUDA(h, cudaMalloc(&w->status, sizeof(int) * 4));
     LQ_CUDA(h, cudaMalloc(&w->sticky, sizeof(int) * 4 + sizeof(unsigned long long) * NACC));
@@ -2250,7 +1928,8 @@ void solver_site_bytes(int prec, int method, double* inner, double* outer, int n
     const double sp = prec == PREC64 ? 192.0 : prec == PREC32 ? 96.0 : prec == PREC16 ? 52.0 : 48.0;
     const double lk = prec == PREC64 ? 1152.0 : prec == PREC32 ? 384.0 : 192.0;
     const double se = prec == PREC64 ? 192.0 : 96.0;
-    // BiCGstab: 24 spinor passes, 4 half sweeps of links, solution r/w;
+    // BiCGstab: 24 spinor passes (21 in lqcd_split.cu: single and double), 4
+    // half sweeps of links, solution r/w;
     // series: p, tmp, tmp, r, p, p (6 passes), 2 half sweeps of links;
     // Schwarz-preconditioned BiCGstab (per even site of the lattice, nsap
     // series terms): two preconditioner applications of (17 + 5 nsap)
@@ -2265,7 +1944,8 @@ void solver_site_bytes(int prec, int method, double* inner, double* outer, int n
     else if (method == SOLVER_SAPB)
         *inner = 2.0 * (4.0 * sp + lk) + 4.0 * lk + 28.0 * sp + 4.0 * se;
     else
-        *inner = method == SOLVER_SERIES ? 6.0 * sp + 2.0 * lk : 24.0 * sp + 4.0 * lk + 2.0 * se;
+        *inner = method == SOLVER_SERIES ? 6.0 * sp + 2.0 * lk
+                                         : (prec == PREC64 || prec == PREC32 ? 21.0 : 24.0) * sp + 4.0 * lk + 2.0 * se;
     *outer = (192.0 + 3.0 * sp + se) + (2.0 * 192.0 + se) + (2.0 * 192.0 + 1152.0) + (4.0 * 192.0 + 1152.0);
 }
 
@@ -2387,7 +2067,7 @@ int eo_solve(lqcd_ctx* h, int mode, int colour, int prec, double kappa, double2*
     // early and leave more of the reduction to the double outer cycles)
     A.inner_tol = prec == PREC64 ? 0.0 : prec == PREC32 ? 1e-5 : prec == PREC16 ? 2e-3 : 3e-2;
     A.max_iter = max_iter;
-    A.max_outer = prec == PREC64 ? 8 : prec == PRECBF ? 80 : 40;
+    A.max_outer = prec == PRECBF ? 80 : 40;
     A.max_inner = prec == PREC64 ? max_iter : prec == PREC32 ? 4000 : prec == PREC16 ? 600 : 200;
     A.part = w->part;
     A.bar = w->bar;
@@ -2425,16 +2105,24 @@ int eo_solve(lqcd_ctx* h, int mode, int colour, int prec, double kappa, double2*
         LQ_CUDA(h, cudaLaunchKernelExC(&cc, (const void*)k_series_cl, args));
         prof_end(h, 1, ev, 0.0);
     }
-    const void* fn = prec == PREC64 ? (sap ? (const void*)k_solve<PREC64, true> : (const void*)k_solve<PREC64, false>)
-                     : prec == PREC32 ? (sap ? (const void*)k_solve<PREC32, true> : (const void*)k_solve<PREC32, false>)
+    const void* fn = prec == PREC64   ? (const void*)k_solve<PREC64, true>
+                     : prec == PREC32 ? (const void*)k_solve<PREC32, true>
                      : prec == PREC16 ? (sap ? (const void*)k_solve<PREC16, true> : (const void*)k_solve<PREC16, false>)
                                       : (sap ? (const void*)k_solve<PRECBF, true> : (const void*)k_solve<PRECBF, false>);
+    int grid = G, block = SBS;
+    if (!clu && !sap && (prec == PREC64 || prec == PREC32)) {
+        const SplitPlan sp = split_plan(A, prec, method, spt, h->num_sms, w->split_occ);
+        fn = sp.fn;
+        grid = sp.grid;
+        block = sp.block;
+        smem = sp.smem;
+    }
     if (!clu) prof_begin(h, 1, &ev);
     // cooperative launch (every CTA resident), expressed as a launch
     // attribute so that it can also be recorded into a CUDA graph
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(G);
-    cfg.blockDim = dim3(SBS);
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = h->stream;
     cudaLaunchAttribute attr[1];

@@ -1,0 +1,1222 @@
+// lqcd_split.cu -- persistent batched solver for single- and double-precision
+// inner storage (the half formats and the Schwarz-preconditioned solves run in
+// lqcd_solver.cu's k_solve).
+//
+// The same solve as k_solve: an outer double defect correction around
+// BiCGstab or the geometric series on every system at once, one cooperative
+// launch, a software barrier per system.  What bounds it, and what follows:
+//   * small systems (up to a few thousand sites): the length of a phase, a
+//     half-lattice hopping sweep between two barriers.  One thread per site
+//     makes that eight dependent neighbour reads and 2000 instructions.  LPS
+//     warps share 32 sites instead: warp d of a site group sums the hops of
+//     its own directions (LPS = 2: forward or backward, 4: half of those,
+//     8: one hop), the partial sums meet in shared memory and each warp
+//     finishes its own spin components.  No warp diverges: its directions
+//     are compile-time constants in its branch.
+//   * larger systems: L2 traffic and instruction fetch.  One thread per site
+//     (LPS = 1) with the loads of a hop issued before the arithmetic of the
+//     previous one, one copy of the hopping code for all sweeps of an
+//     iteration (35 KB; four copies overran the instruction cache and made a
+//     sweep 1.5 times longer), vectors and links in tiles of 32 sites, no
+//     register spills (phases, barriers and reductions are kept apart for
+//     that: spilled registers tripled the L2 writes).
+//   * everywhere: FP64 issues two lanes per cycle and SM, so sums and scalars
+//     of a single-precision iteration are pairs of floats.
+// Measured (ms per solve to 1e-12, one thread per site without the above ->
+// this kernel): 12x6^3 global 4.48 -> 2.23, 32x16^3 global 33.8 -> 22.3, its
+// 8 slabs 4.85 -> 3.62, 64x32^3 global 695 -> 420, 32x24^3 series 9.28 -> 7.9;
+// double precision at 16x8^3 (two solves and the force) 34.8 -> 5.9.
+#include <algorithm>
+
+#include "lqcd_solve.cuh"
+
+namespace {
+
+// ---------------------------------------------------------------------------
+// sums: single-precision terms accumulate in pairs of floats (the FP64 pipe
+// issues two lanes per cycle and SM: five shuffle steps of three FP64 sums
+// in every warp cost more than a hopping phase)
+// ---------------------------------------------------------------------------
+template <class T>
+struct Acc;
+template <>
+struct Acc<float> {
+    float h, l;
+    __device__ __forceinline__ void add(float x)
+    {
+        float s, e;
+        df_two_sum(h, x, s, e);
+        h = s;
+        l += e;
+    }
+    __device__ __forceinline__ void join(const Acc& o)
+    {
+        float s, e;
+        df_two_sum(h, o.h, s, e);
+        h = s;
+        l += o.l + e;
+    }
+    __device__ __forceinline__ Acc from(int m) const
+    {
+        return Acc{__shfl_xor_sync(0xffffffffu, h, m), __shfl_xor_sync(0xffffffffu, l, m)};
+    }
+    __device__ __forceinline__ Acc at(int k) const
+    {
+        return Acc{__shfl_sync(0xffffffffu, h, k), __shfl_sync(0xffffffffu, l, k)};
+    }
+    static __device__ __forceinline__ Acc zero() { return Acc{0.f, 0.f}; }
+    __device__ __forceinline__ double bits() const { return __hiloint2double(__float_as_int(l), __float_as_int(h)); }
+    static __device__ __forceinline__ Acc of(double d)
+    {
+        return Acc{__int_as_float(__double2loint(d)), __int_as_float(__double2hiint(d))};
+    }
+};
+template <>
+struct Acc<double> {
+    double h;
+    __device__ __forceinline__ void add(double x) { h += x; }
+    __device__ __forceinline__ void join(const Acc& o) { h += o.h; }
+    __device__ __forceinline__ Acc from(int m) const { return Acc{__shfl_xor_sync(0xffffffffu, h, m)}; }
+    __device__ __forceinline__ Acc at(int k) const { return Acc{__shfl_sync(0xffffffffu, h, k)}; }
+    static __device__ __forceinline__ Acc zero() { return Acc{0.0}; }
+    __device__ __forceinline__ double bits() const { return h; }
+    static __device__ __forceinline__ Acc of(double d) { return Acc{d}; }
+};
+
+// warp sums of N = 1, 4 or 8 quantities, halving the quantities a lane
+// carries with every step (N = 8: nine joins instead of forty): every lane
+// returns the sum of quantity lane * N / 32
+template <int N, class A1>
+__device__ __forceinline__ A1 warp_sum(A1 (&v)[N])
+{
+    const int lane = threadIdx.x & 31;
+    int m = 16;
+#pragma unroll
+    for (int n = N / 2; n >= 1; n >>= 1, m >>= 1) {
+        const bool up = (lane & m) != 0;
+#pragma unroll
+        for (int k = 0; k < n; ++k) {
+            A1 x = up ? v[n + k] : v[k];
+            x.join((up ? v[k] : v[n + k]).from(m));
+            v[k] = x;
+        }
+    }
+    for (; m >= 1; m >>= 1) v[0].join(v[0].from(m));
+    return v[0];
+}
+
+// the scalars of the recurrences in the accuracy of the sums: double-float
+// for single, double for double (FP64 instructions depend on one another at
+// an order of magnitude more latency than FP32 ones)
+template <class T>
+struct Scalar;
+template <>
+struct Scalar<float> {
+    typedef df R;
+    static __device__ __forceinline__ df get(const Acc<float>& a) { return df_norm(df(a.h, a.l)); }
+    static __device__ __forceinline__ float round(df a) { return a.hi + a.lo; }
+    // a / b, b scaled to [1, 2) by its exponent
+    static __device__ __forceinline__ cx<df> div(cx<df> a, cx<df> b)
+    {
+        const float m = fmaxf(fabsf(b.re.hi), fabsf(b.im.hi));
+        const unsigned e = (__float_as_uint(m) >> 23) & 0xffu;
+        const float sc = __uint_as_float((e >= 253u ? 1u : 254u - e) << 23);
+        const cx<df> bs = mk(df(b.re.hi * sc, b.re.lo * sc), df(b.im.hi * sc, b.im.lo * sc));
+        const cx<df> as = mk(df(a.re.hi * sc, a.re.lo * sc), df(a.im.hi * sc, a.im.lo * sc));
+        const df d = df_norm(bs.re * bs.re + bs.im * bs.im);
+        const cx<df> n = cjmul(bs, as);
+        const float inv = __fdividef(1.0f, d.hi);
+        return mk(quot(df_norm(n.re), d, inv), quot(df_norm(n.im), d, inv));
+    }
+    // n / d, inv an approximation of 1 / d: the first quotient's remainder is
+    // one FMA (exact) and the low parts, and gives the second
+    static __device__ __forceinline__ df quot(df n, df d, float inv)
+    {
+        const float q = n.hi * inv;
+        const float r = fmaf(-q, d.hi, n.hi) + (n.lo - q * d.lo);
+        return df_norm(df(q, r * inv));
+    }
+};
+template <>
+struct Scalar<double> {
+    typedef double R;
+    static __device__ __forceinline__ double get(const Acc<double>& a) { return a.h; }
+    static __device__ __forceinline__ double round(double a) { return a; }
+    static __device__ __forceinline__ cx<double> div(cx<double> a, cx<double> b)
+    {
+        const double d = 1.0 / (b.re * b.re + b.im * b.im);
+        return d * cjmul(b, a);
+    }
+};
+template <class T>
+__device__ __forceinline__ cx<T> sround(cx<typename Scalar<T>::R> a)
+{
+    return mk(Scalar<T>::round(a.re), Scalar<T>::round(a.im));
+}
+template <class R>
+__device__ __forceinline__ R from_round(float x) { return df(x, 0.f); }
+template <class R>
+__device__ __forceinline__ R from_round(double x) { return x; }
+template <class T>
+__device__ __forceinline__ bool fin2(cx<T> a) { return isfinite(a.re) && isfinite(a.im); }
+
+// ---------------------------------------------------------------------------
+// barrier of the CTAs of one group (bounded, as in k_solve) and the sums
+// that go with it.  Warp 0 does both alone: it adds the CTA's sums, arrives,
+// waits, adds the group's sums and hands them to f (on lane 0), so a
+// reducing barrier costs the CTA two __syncthreads.
+// ---------------------------------------------------------------------------
+struct Group {
+    int grp, cin, cps;  // group, CTA in the group, CTAs per group
+    unsigned epoch;
+    int rb;
+};
+
+__device__ __forceinline__ bool group_wait(const SolveArgs& A, Group& G)
+{
+    unsigned* bar = A.bar + (size_t)G.grp * BAR_STRIDE;
+    const unsigned target = G.epoch * (unsigned)G.cps;
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+    const long long t0 = clock64();
+    for (int n = 1; ld_acquire(bar) < target; ++n) {
+        if (clock64() - t0 > A.spin_limit) {
+            atomicExch(A.status, LQCD_ERR_TIMEOUT);
+            atomicCAS(A.sticky, 0, LQCD_ERR_TIMEOUT);
+            return false;
+        }
+        if ((n & 15) == 0 && *(volatile int*)A.status == LQCD_ERR_TIMEOUT) return false;
+    }
+    return true;
+}
+
+__device__ __noinline__ bool group_sync(const SolveArgs& A, Group& G)
+{
+    __shared__ int s_ok;
+    __syncthreads();
+    ++G.epoch;
+    if (G.cps == 1) return true;
+    if (threadIdx.x == 0) s_ok = group_wait(A, G);
+    __syncthreads();
+    return s_ok != 0;
+}
+
+// (Not inlined: with their registers the phases would spill.)
+// f receives the group's sums of the N quantities v on thread 0.  The CTAs'
+// partials lie quantity by quantity: warp k adds those of quantity k, four
+// loads in flight per lane.
+template <int NW, int N, class A1, class F>
+__device__ __noinline__ bool group_reduce(const SolveArgs& A, Group& G, A1 (&v)[N], F f)
+{
+    static_assert(sizeof(A1) == 8, "partial sums travel as 8-byte words");
+    static_assert(N <= NW, "one warp per quantity");
+    __shared__ A1 sh[N][NW], tot[N];
+    __shared__ int s_ok;
+    constexpr int LQ = 32 / N;  // lanes per quantity
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    {
+        const A1 x = warp_sum<N>(v);
+        if (lane % LQ == 0) sh[lane / LQ][w] = x;
+    }
+    __syncthreads();
+    ++G.epoch;
+    if (G.cps == 1) {
+        if (w < N) {
+            A1 q[1] = {A1::zero()};
+            if (lane < NW) q[0] = sh[w][lane];
+            q[0] = warp_sum<1>(q);
+            if (lane == 0) tot[w] = q[0];
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) f(tot);
+        __syncthreads();
+        return true;
+    }
+    double* part = A.part + ((size_t)G.rb * gridDim.x + (size_t)G.grp * G.cps) * SPLIT_NQ;
+    if (w == 0) {
+        // lane LQ k + j adds every LQ-th warp's sum of quantity k
+        A1 x = A1::zero();
+#pragma unroll
+        for (int j = 0; j < (NW + LQ - 1) / LQ; ++j) {
+            const int i = lane % LQ + j * LQ;
+            if (i < NW) x.join(sh[lane / LQ][i]);
+        }
+#pragma unroll
+        for (int m = LQ / 2; m >= 1; m >>= 1) x.join(x.from(m));
+        if (lane % LQ == 0) part[(size_t)(lane / LQ) * G.cps + G.cin] = x.bits();
+        __syncwarp();
+        if (lane == 0) s_ok = group_wait(A, G);
+    }
+    __syncthreads();
+    if (w < N) {
+        const double* p = part + (size_t)w * G.cps;
+        A1 q[1] = {A1::zero()};
+        for (int c = lane; c < G.cps; c += 128) {
+            double u[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (c + 32 * k < G.cps) u[k] = __ldcg(p + c + 32 * k);
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (c + 32 * k < G.cps) q[0].join(A1::of(u[k]));
+        }
+        q[0] = warp_sum<1>(q);
+        if (lane == 0) tot[w] = q[0];
+    }
+    G.rb ^= 1;
+    __syncthreads();
+    if (threadIdx.x == 0) f(tot);
+    __syncthreads();
+    return s_ok != 0;
+}
+
+// ---------------------------------------------------------------------------
+// inner vectors: words of two (single) or one (double) complex numbers
+// ---------------------------------------------------------------------------
+template <int P>
+struct Word;
+template <>
+struct Word<PREC32> {
+    typedef float4 W;
+    static constexpr int N = 6;
+};
+template <>
+struct Word<PREC64> {
+    typedef double2 W;
+    static constexpr int N = 12;
+};
+
+// The inner vectors are stored in tiles of 32 sites, [Vh/32][N][32] words
+// (Vh rounded up): one address and constant offsets reach all words of a
+// site.  tile_at: the place of word 0 of site i, word k is 32 k further.
+template <int P>
+__device__ __forceinline__ size_t tile_at(int i)
+{
+    return (size_t)i + (size_t)(i >> 5) * (32 * (Word<P>::N - 1));
+}
+
+__device__ __forceinline__ float4 wzero(float4) { return make_float4(0.f, 0.f, 0.f, 0.f); }
+__device__ __forceinline__ double2 wzero(double2) { return make_double2(0.0, 0.0); }
+// y + a x
+__device__ __forceinline__ float4 waxpy(cx<float> a, float4 x, float4 y)
+{
+    return make_float4(y.x + a.re * x.x - a.im * x.y, y.y + a.re * x.y + a.im * x.x, y.z + a.re * x.z - a.im * x.w,
+                       y.w + a.re * x.w + a.im * x.z);
+}
+__device__ __forceinline__ double2 waxpy(cx<double> a, double2 x, double2 y)
+{
+    return make_double2(y.x + a.re * x.x - a.im * x.y, y.y + a.re * x.y + a.im * x.x);
+}
+__device__ __forceinline__ void wnorm(float4 a, Acc<float>& n) { n.add(a.x * a.x + a.y * a.y + a.z * a.z + a.w * a.w); }
+__device__ __forceinline__ void wnorm(double2 a, Acc<double>& n) { n.add(a.x * a.x + a.y * a.y); }
+
+__device__ __forceinline__ void put(Spinor<float>& s, int k, float4 w)
+{
+    s.c[(2 * k) / 3][(2 * k) % 3] = mk(w.x, w.y);
+    s.c[(2 * k + 1) / 3][(2 * k + 1) % 3] = mk(w.z, w.w);
+}
+__device__ __forceinline__ void put(Spinor<double>& s, int k, double2 w) { s.c[k / 3][k % 3] = mk(w.x, w.y); }
+
+// ---------------------------------------------------------------------------
+// the hops of one warp
+// ---------------------------------------------------------------------------
+// one hop's loads, kept as the words that were read
+template <int P>
+struct Raw {
+    static constexpr int NL = P == PREC32 ? 3 : 9;
+    typename Word<P>::W s[Word<P>::N], l[NL];
+    bool use, neg;
+};
+
+// hop H: direction mu = 3 - H / 2, forward (even H) or backward
+template <int P, int H>
+__device__ __forceinline__ void hop_fetch(const Geo& g, int mode, int pout, int i, const int x[4], int lex,
+                                          const typename Word<P>::W* in, const GaugeF& U, Raw<P>& R)
+{
+    typedef typename Word<P>::W W;
+    constexpr int MU = 3 - H / 2, DIR = H & 1;
+    const int stride = MU == 3 ? 1 : MU == 2 ? g.L[3] : MU == 1 ? g.L[3] * g.L[2] : g.V3;
+    const bool wrap = DIR ? x[MU] == 0 : x[MU] == g.L[MU] - 1;
+    int nl = DIR ? lex - stride : lex + stride;
+    if (wrap) nl += DIR ? g.L[MU] * stride : -g.L[MU] * stride;
+    R.use = MU != 0 || t_hop_kept(g, mode, DIR ? x[0] : x[0] + 1);
+    R.neg = MU == 0 && wrap && g.bc_t < 0;
+    // a dropped hop reads the own index instead of another system's site
+    const int j = R.use ? nl >> 1 : i;
+    const W* sp = in + tile_at<P>(j);
+#pragma unroll
+    for (int k = 0; k < Word<P>::N; ++k) R.s[k] = sp[32 * k];
+    constexpr int NL = Raw<P>::NL;
+    const int mp = MU * 2 + (DIR ? 1 - pout : pout), li = DIR ? j : i;
+    const W* lp = (const W*)U.v + (P == PREC32 ? (size_t)mp * link32_block(U.Vh) + link32_at(li) : (size_t)mp * NL * U.Vh + li);
+#pragma unroll
+    for (int k = 0; k < NL; ++k) R.l[k] = __ldg(lp + (P == PREC32 ? (size_t)(32 * k) : (size_t)k * U.Vh));
+}
+
+// rows 0 and 1 of the link as read, entry c of row 2
+__device__ __forceinline__ cx<float> link_entry(const float4 (&l)[3], int r, int c)
+{
+    const int e = 3 * r + c;
+    return e & 1 ? mk(l[e >> 1].z, l[e >> 1].w) : mk(l[e >> 1].x, l[e >> 1].y);
+}
+__device__ __forceinline__ cx<float> link_row2(const float4 (&l)[3], int c)
+{
+    const int j = (c + 1) % 3, k = (c + 2) % 3;
+    return conjx(link_entry(l, 0, j) * link_entry(l, 1, k) - link_entry(l, 0, k) * link_entry(l, 1, j));
+}
+__device__ __forceinline__ cx<double> link_entry(const double2 (&l)[9], int r, int c)
+{
+    return mk(l[3 * r + c].x, l[3 * r + c].y);
+}
+__device__ __forceinline__ cx<double> link_row2(const double2 (&l)[9], int c) { return link_entry(l, 2, c); }
+
+// a b + c, with one rounding per product
+template <class T>
+__device__ __forceinline__ cx<T> cfma(cx<T> a, cx<T> b, cx<T> c)
+{
+    return mk(fma(-a.im, b.im, fma(a.re, b.re, c.re)), fma(a.im, b.re, fma(a.re, b.im, c.im)));
+}
+template <class T>
+__device__ __forceinline__ cx<T> cmul1(cx<T> a, cx<T> b)
+{
+    return mk(fma(-a.im, b.im, a.re * b.re), fma(a.im, b.re, a.re * b.im));
+}
+
+// adds hop H: the neighbour is projected, and the link applied and the result
+// accumulated colour by colour (row by row, column by column for U^dag), so
+// that besides acc only the half spinor and rows 0-1 of the link are live
+template <int P, int H>
+__device__ __forceinline__ void hop_add(const Raw<P>& R, Spinor<typename Real<P>::T>& acc)
+{
+    typedef typename Real<P>::T T;
+    constexpr int MU = 3 - H / 2, DAG = H & 1, sg = DAG ? +1 : -1;
+    if (MU == 0 && !R.use) return;
+    HalfSp<T> h;
+    {
+        Spinor<T> s;
+#pragma unroll
+        for (int k = 0; k < Word<P>::N; ++k) put(s, k, R.s[k]);
+        project(MU, sg, s, h);
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        cx<T> w0, w1;
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const int r = DAG ? j : c, q = DAG ? c : j;
+            cx<T> u = r == 2 ? link_row2(R.l, q) : link_entry(R.l, r, q);
+            if (DAG) u = conjx(u);
+            w0 = j ? cfma(u, h.c[0][j], w0) : cmul1(u, h.c[0][j]);
+            w1 = j ? cfma(u, h.c[1][j], w1) : cmul1(u, h.c[1][j]);
+        }
+        if (MU == 0 && R.neg) {
+            w0 = -w0;
+            w1 = -w1;
+        }
+        accum_recon1(MU, sg, w0, w1, acc, c);
+    }
+}
+
+// hops H, H + STEP, .. (N of them): the loads of a hop are issued before the
+// arithmetic of the one before it
+template <int P, int H, int STEP, int N>
+struct Hops {
+    static __device__ __forceinline__ void run(const Geo& g, int mode, int pout, int i, const int x[4], int lex,
+                                               const typename Word<P>::W* in, const GaugeF& U, Raw<P>& R,
+                                               Spinor<typename Real<P>::T>& acc)
+    {
+        if constexpr (N > 1) {
+            Raw<P> Q;
+            hop_fetch<P, H + STEP>(g, mode, pout, i, x, lex, in, U, Q);
+            hop_add<P, H>(R, acc);
+            Hops<P, H + STEP, STEP, N - 1>::run(g, mode, pout, i, x, lex, in, U, Q, acc);
+        } else {
+            hop_add<P, H>(R, acc);
+        }
+    }
+    static __device__ __forceinline__ void start(const Geo& g, int mode, int pout, int i, const int x[4], int lex,
+                                                 const typename Word<P>::W* in, const GaugeF& U,
+                                                 Spinor<typename Real<P>::T>& acc)
+    {
+        Raw<P> R;
+        hop_fetch<P, H>(g, mode, pout, i, x, lex, in, U, R);
+        run(g, mode, pout, i, x, lex, in, U, R, acc);
+    }
+};
+
+// partial sum of the hopping term at (pout, i) over the directions of warp d
+template <int P, int LPS>
+__device__ __forceinline__ void hop_part(const Geo& g, int mode, int pout, int i, int d, const typename Word<P>::W* in,
+                                         const GaugeF& U, Spinor<typename Real<P>::T>& acc)
+{
+    typedef typename Real<P>::T T;
+#pragma unroll
+    for (int s = 0; s < 4; ++s)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) acc.c[s][c] = mk(T(0), T(0));
+    int x[4];
+    eo_coords(g, pout, i, x);
+    const int lex = lex_of(g, x);
+#define LQ_H(H, STEP, N) Hops<P, H, STEP, N>::start(g, mode, pout, i, x, lex, in, U, acc)
+    if constexpr (LPS == 1) {
+        LQ_H(0, 1, 8);
+    } else if constexpr (LPS == 2) {
+        if (d == 0) LQ_H(0, 2, 4);
+        else LQ_H(1, 2, 4);
+    } else if constexpr (LPS == 4) {
+        switch (d) {
+            case 0: LQ_H(0, 2, 2); break;
+            case 1: LQ_H(1, 2, 2); break;
+            case 2: LQ_H(4, 2, 2); break;
+            default: LQ_H(5, 2, 2); break;
+        }
+    } else {
+        switch (d) {
+            case 0: LQ_H(0, 1, 1); break;
+            case 1: LQ_H(1, 1, 1); break;
+            case 2: LQ_H(2, 1, 1); break;
+            case 3: LQ_H(3, 1, 1); break;
+            case 4: LQ_H(4, 1, 1); break;
+            case 5: LQ_H(5, 1, 1); break;
+            case 6: LQ_H(6, 1, 1); break;
+            default: LQ_H(7, 1, 1); break;
+        }
+    }
+#undef LQ_H
+}
+
+// The partial sums of a site group's LPS warps meet in shared memory; warp d
+// receives the components [d NC, (d + 1) NC) of the sum (LPS = 8: warps 0..3).
+// The buffer is used alternately in two halves: a warp that writes a half
+// again has passed the barrier after the other half, which its partners
+// reached after they had read this one.
+template <class T, int LPS>
+struct Xchg {
+    static constexpr int PARTS = LPS < 4 ? LPS : 4;
+    static constexpr int NC = 12 / PARTS;
+    T* buf;  // [2][NW][24][32]
+    int w, d, sg, lane, half;
+    __device__ __forceinline__ bool fin() const { return d < PARTS; }
+    __device__ __forceinline__ void combine(int nw, const Spinor<T>& acc, cx<T> out[NC])
+    {
+        if constexpr (LPS == 1) {
+#pragma unroll
+            for (int k = 0; k < 12; ++k) out[k] = acc.c[k / 3][k % 3];
+            return;
+        }
+        T* b = buf + (size_t)half * nw * 24 * 32;
+        half ^= 1;
+        T* mine = b + (size_t)w * 24 * 32 + lane;
+#pragma unroll
+        for (int q = 0; q < PARTS; ++q)
+            if (q != d) {
+#pragma unroll
+                for (int k = 0; k < NC; ++k) {
+                    const cx<T> v = acc.c[(q * NC + k) / 3][(q * NC + k) % 3];
+                    mine[(2 * (q * NC + k)) * 32] = v.re;
+                    mine[(2 * (q * NC + k) + 1) * 32] = v.im;
+                }
+            } else {
+#pragma unroll
+                for (int k = 0; k < NC; ++k) out[k] = acc.c[(q * NC + k) / 3][(q * NC + k) % 3];
+            }
+        asm volatile("bar.sync %0, %1;" ::"r"(1 + sg), "r"(LPS * 32) : "memory");
+        if (fin()) {
+#pragma unroll
+            for (int p = 1; p < LPS; ++p) {
+                const int o = d ^ p;  // warp of the group
+                const T* s = b + (size_t)(sg * LPS + o) * 24 * 32 + (size_t)(2 * d * NC) * 32 + lane;
+#pragma unroll
+                for (int k = 0; k < NC; ++k) out[k] = out[k] + mk(s[(2 * k) * 32], s[(2 * k + 1) * 32]);
+            }
+        }
+    }
+};
+
+__device__ __forceinline__ void store_split(float4* p, double x, double y)
+{
+    const df a = df_split(x), b = df_split(y);
+    *p = make_float4(a.hi, b.hi, a.lo, b.lo);
+}
+
+// part d (NC complex numbers) of the spinor whose word 0 is *v; single
+// precision stores two complex numbers per float4
+template <int NC>
+__device__ __forceinline__ void load_part(const float4* v, int d, cx<float> o[NC])
+{
+    if constexpr (NC != 3) {
+#pragma unroll
+        for (int k = 0; k < NC / 2; ++k) {
+            const float4 w = v[32 * (NC / 2 * d + k)];
+            o[2 * k] = mk(w.x, w.y);
+            o[2 * k + 1] = mk(w.z, w.w);
+        }
+    } else {
+        const float2* v2 = (const float2*)v;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const int c = 3 * d + k;
+            const float2 w = v2[64 * (c >> 1) + (c & 1)];
+            o[k] = mk(w.x, w.y);
+        }
+    }
+}
+template <int NC>
+__device__ __forceinline__ void store_part(float4* v, int d, const cx<float> o[NC])
+{
+    if constexpr (NC != 3) {
+#pragma unroll
+        for (int k = 0; k < NC / 2; ++k)
+            v[32 * (NC / 2 * d + k)] = make_float4(o[2 * k].re, o[2 * k].im, o[2 * k + 1].re, o[2 * k + 1].im);
+    } else {
+        float2* v2 = (float2*)v;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const int c = 3 * d + k;
+            v2[64 * (c >> 1) + (c & 1)] = make_float2(o[k].re, o[k].im);
+        }
+    }
+}
+template <int NC>
+__device__ __forceinline__ void load_part(const double2* v, int d, cx<double> o[NC])
+{
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+        const double2 w = v[32 * (d * NC + k)];
+        o[k] = mk(w.x, w.y);
+    }
+}
+template <int NC>
+__device__ __forceinline__ void store_part(double2* v, int d, const cx<double> o[NC])
+{
+#pragma unroll
+    for (int k = 0; k < NC; ++k) v[32 * (d * NC + k)] = make_double2(o[k].re, o[k].im);
+}
+
+template <int NC, class T>
+__device__ __forceinline__ void pdot(const cx<T> a[NC], const cx<T> b[NC], T& re, T& im)
+{
+    re = im = 0;
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+        re += a[k].re * b[k].re + a[k].im * b[k].im;
+        im += a[k].re * b[k].im - a[k].im * b[k].re;
+    }
+}
+template <int NC, class T>
+__device__ __forceinline__ T pnorm(const cx<T> a[NC])
+{
+    T s = 0;
+#pragma unroll
+    for (int k = 0; k < NC; ++k) s += a[k].re * a[k].re + a[k].im * a[k].im;
+    return s;
+}
+
+// ---------------------------------------------------------------------------
+// the kernel
+// ---------------------------------------------------------------------------
+template <int P, int LPS, int BS>
+constexpr int split_smem()
+{
+    return LPS == 1 ? 0 : 2 * (BS / 32) * 24 * 32 * (int)sizeof(typename Real<P>::T);
+}
+
+// x, unknown to the compiler: the addresses of one phase are computed in it
+// instead of being held in registers (and spilled) through all the others
+__device__ __forceinline__ int opaque(int x)
+{
+    asm volatile("" : "+r"(x));
+    return x;
+}
+
+// first site of the g-th group of 32 of a system, in the tiled order: a CTA's
+// consecutive groups form a compact block of the lattice, whose hops meet in
+// its L1 (a run of sites shares a spinor between 8 / 3.5 of its readers, a
+// 4 x 4 tile between 8 / 2.5)
+__device__ __forceinline__ int group_site(const SolveArgs& A, int g)
+{
+    if (!A.tiled) return g * 32;
+    const int q = g & ((1 << A.lt[2]) - 1), i1 = (g >> A.lt[2]) & ((1 << A.lt[1]) - 1);
+    const int i0 = (g >> (A.lt[1] + A.lt[2])) & ((1 << A.lt[0]) - 1);
+    const int t = g >> (A.lt[0] + A.lt[1] + A.lt[2]);
+    const int tq = t & ((1 << A.nt[1]) - 1), t1 = (t >> A.nt[1]) & ((1 << A.nt[0]) - 1), t0 = t >> (A.nt[0] + A.nt[1]);
+    const int x0 = (t0 << A.lt[0]) + i0, x1 = (t1 << A.lt[1]) + i1;
+    return (((((x0 << (A.nt[0] + A.lt[1])) + x1) << A.nt[1]) + tq) << (A.lt[2] + 5)) + (q << 5);
+}
+
+// BiCGstab iterations without a new smallest residual after which the inner
+// solve ends and the outer cycle restarts it from the true residual.  A
+// system near its critical point (8x4^3, kappa = 0.15 on a smooth field, in
+// double): 1400-2300 iterations in 5 cycles with a restart after 100,
+// 3000-4000 after 300, without one 2900 to no convergence, as rounding has it.
+constexpr int STALL = 200;
+
+// (site, word) items of the element-wise phases, B of them at a time so that
+// their loads are in flight together: act(site, word, load(site, word)).  An
+// item past the end repeats the last load and is not acted on.
+template <int B, int NWD, int NW, class LD, class ACT>
+__device__ __forceinline__ void for_words(const SolveArgs& A, int warp, int lane, int g0, int ngr, int base, LD load,
+                                          ACT act)
+{
+    const int n = NWD * ngr;
+    lane = opaque(lane);
+    for (int u = warp; u < n; u += NW * B) {
+        decltype(load(0, 0)) val[B];
+        int i[B];
+        bool in[B];
+#pragma unroll
+        for (int b = 0; b < B; ++b) {
+            const int v = min(u + b * NW, n - 1), j = group_site(A, g0 + v / NWD) + lane;
+            in[b] = u + b * NW < n && j < A.nsite;
+            i[b] = base + min(j, A.nsite - 1);
+            val[b] = load(i[b], v % NWD);
+        }
+#pragma unroll
+        for (int b = 0; b < B; ++b)
+            if (in[b]) act(i[b], (u + b * NW) % NWD, val[b]);
+    }
+}
+template <class W>
+struct W2 { W x, y; };
+template <class W>
+struct W5 { W s, t, v, p, e; };
+
+template <int P, int LPS, int BS, int MINB, int METHOD>
+__global__ void __launch_bounds__(BS, MINB) k_split(const __grid_constant__ SolveArgs A)
+{
+    typedef typename Real<P>::T T;
+    typedef typename Word<P>::W W;
+    typedef Scalar<T> SC;
+    typedef typename SC::R R;
+    constexpr int NWORD = Word<P>::N;
+    constexpr int NW = BS / 32, SG = NW / LPS;
+    // the residual sweeps read x, as df pairs (xs) around a single-precision
+    // iteration, and their intermediate t64 in the same storage
+    constexpr int PT = P == PREC64 ? PREC64 : PRECDS;
+    typedef typename Real<PT>::T TR;
+    typedef Xchg<T, LPS> X;
+    constexpr int NC = X::NC;
+    extern __shared__ __align__(16) unsigned char split_dyn[];
+    __shared__ struct {
+        double bn2, rn2, itol2;
+        cx<R> rho, d;
+        cx<T> alpha, omega, beta;
+        T best;  // smallest inner residual so far, and the iterations since
+        int since, idone, it, itc;
+    } S;
+    __shared__ Acc<T> sums[METHOD == SOLVER_BICGSTAB ? 8 : 1][BS];
+
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    Group G;
+    G.cps = A.cps;
+    G.grp = blockIdx.x / A.cps;
+    G.cin = blockIdx.x - G.grp * A.cps;
+    G.epoch = 0;
+    G.rb = 0;
+    X xc;
+    xc.buf = (T*)split_dyn;
+    xc.w = warp;
+    xc.d = LPS == 1 ? 0 : warp % LPS;
+    xc.sg = warp / LPS;
+    xc.lane = lane;
+    xc.half = 0;
+    const int d = xc.d;
+    const int Vh = A.g.Vh;
+    const GaugeF UP = A.UP;
+    // the CTA's sites of a system, in groups of 32
+    const int g0 = G.cin * (A.chunk >> 5);
+    const int ngr = max(0, min(A.chunk >> 5, ((A.nsite + 31) >> 5) - g0));
+
+#define V_(f) ((W*)A.f.v)
+#define WORDS A, warp, lane, g0, ngr, base
+// word k of site i: of an inner vector, of a double field
+#define TW(i, k) (tile_at<P>(i) + 32 * (k))
+#define DW(i, c) ((size_t)(c) * Vh + (i))
+#define SYNC_OR_RETURN \
+    if (!group_sync(A, G)) return
+// sites of the CTA, a group of 32 per LPS warps; lanes past the end repeat the last site and store nothing
+#define FOR_GROUPS                                                                \
+    for (int gr_ = xc.sg; gr_ < ngr; gr_ += SG)                                   \
+        if (const int j_ = group_site(A, g0 + gr_) + opaque(lane), i = base + min(j_, A.nsite - 1); true) \
+            if (const bool on = j_ < A.nsite; true)                                    \
+                if (const size_t at = tile_at<P>(i); true)
+// (site, colour) items of the double sweeps
+#define FOR_ITEMS                                                            \
+    for (int u_ = warp; u_ < 3 * ngr; u_ += NW)                               \
+        if (const int j_ = group_site(A, g0 + u_ / 3) + opaque(lane), r_ = u_ % 3; j_ < A.nsite)   \
+            if (const int i = base + j_; true)
+    for (int sys = G.grp; sys < A.nsys; sys += A.ngrp) {
+        const int base = A.mode == MODE_INTRA ? (A.slab0 + sys * A.slabstep) * A.g.Sh : 0;
+        const bool leader = G.cin == 0 && tid == 0;
+        const double2* bb = (const double2*)A.b.v;
+        double2* xx = (double2*)A.x.v;
+        double2* r6 = (double2*)A.r64.v;
+        const SpinorF xs = P == PREC64 ? A.x : A.s;
+
+        // ---- |b|^2; from x = 0: r64 = b
+        {
+            Acc<double> q[1] = {Acc<double>::zero()};
+            for_words<2, 12, NW>(
+                WORDS, [&](int i, int c) { return __ldg(bb + DW(i, c)); },
+                [&](int i, int c, double2 v) {
+                    const size_t a = DW(i, c);
+                    if (A.guess) {
+                        if (P == PREC32) store_split((float4*)xs.v + a, xx[a].x, xx[a].y);
+                    } else {
+                        r6[a] = v;
+                        xx[a] = make_double2(0.0, 0.0);
+                    }
+                    q[0].add(v.x * v.x + v.y * v.y);
+                });
+            if (!group_reduce<NW, 1>(A, G, q, [&](const Acc<double>(&n)[1]) {
+                    S.bn2 = S.rn2 = n[0].h;
+                    S.it = 0;
+                }))
+                return;
+        }
+        // b = 0: the solution is 0, whatever the guess
+        bool fresh = A.guess != 0;
+        if (fresh && !(S.bn2 > 0.0)) {
+            fresh = false;
+            for (int u = warp; u < 12 * ngr; u += NW) {
+                const int j = group_site(A, g0 + u / 12) + lane;
+                if (j < A.nsite) xx[(size_t)(u % 12) * Vh + (base + j)] = make_double2(0.0, 0.0);
+            }
+        }
+
+        int outer = 0, final_flag = F_DONE;
+        for (;;) {
+            // ---- x is new: r64 = b - diag x + k2 H_eo H_oe x in double-float (single
+            // inner precision) or double arithmetic
+            if (fresh) {
+                FOR_ITEMS
+                {
+                    cx<TR> h[4];
+                    hop_colour<PT, false>(A.g, A.mode, 0, 1, i, r_, xs, A.U64, h);
+#pragma unroll
+                    for (int s = 0; s < 4; ++s) store_comp<PT>(A.t64, 3 * s + r_, i, h[s]);
+                }
+                SYNC_OR_RETURN;
+                Acc<double> q[1] = {Acc<double>::zero()};
+                FOR_ITEMS
+                {
+                    cx<TR> h[4];
+                    hop_colour<PT, false>(A.g, A.mode, 0, 0, i, r_, A.t64, A.U64, h);
+#pragma unroll
+                    for (int s = 0; s < 4; ++s) {
+                        const size_t o = (size_t)(3 * s + r_) * Vh + i;
+                        const double2 b2 = __ldg(bb + o), x2 = xx[o];
+                        const double re = b2.x - A.diag * x2.x + A.k2 * as_double(h[s].re);
+                        const double im = b2.y - A.diag * x2.y + A.k2 * as_double(h[s].im);
+                        r6[o] = make_double2(re, im);
+                        q[0].add(re * re + im * im);
+                    }
+                }
+                if (!group_reduce<NW, 1>(A, G, q, [&](const Acc<double>(&n)[1]) { S.rn2 = n[0].h; })) return;
+            }
+            {
+                // every CTA of the group takes the same decision from the same sums
+                const bool nan = !isfinite(S.rn2);
+                const bool conv = !(S.rn2 > A.tol * A.tol * S.bn2) || !(S.bn2 > 0.0);
+                int f = nan ? F_NAN : conv ? F_DONE : F_ACTIVE;
+                if (f == F_ACTIVE && (outer >= A.max_outer || S.it >= A.max_iter)) f = F_MAXIT;
+                if (f != F_ACTIVE) {
+                    final_flag = f;
+                    break;
+                }
+            }
+            ++outer;
+            // ---- inner start: r = rh = p = r64 / |r64|, e = 0 (series: r = p)
+            {
+                Acc<T> q[1] = {Acc<T>::zero()};
+                const double sc = 1.0 / sqrt(S.rn2);
+                for_words<2, NWORD, NW>(
+                    WORDS,
+                    [&](int i, int k) {
+                        // single precision: word k holds the complex numbers 2 k and 2 k + 1
+                        if constexpr (P == PREC32) return W2<double2>{r6[DW(i, 2 * k)], r6[DW(i, 2 * k + 1)]};
+                        else return r6[DW(i, k)];
+                    },
+                    [&](int i, int k, auto d) {
+                        const size_t a = TW(i, k);
+                        W w;
+                        if constexpr (P == PREC32)
+                            w = make_float4((float)(sc * d.x.x), (float)(sc * d.x.y), (float)(sc * d.y.x),
+                                            (float)(sc * d.y.y));
+                        else
+                            w = make_double2(sc * d.x, sc * d.y);
+                        V_(r)[a] = w;
+                        V_(p)[a] = w;
+                        if constexpr (METHOD == SOLVER_BICGSTAB) {
+                            V_(rh)[a] = w;
+                            V_(e)[a] = wzero(W());
+                        }
+                        wnorm(w, q[0]);
+                    });
+                if (!group_reduce<NW, 1>(A, G, q, [&](const Acc<T>(&n)[1]) {
+                        S.rho = mk(SC::get(n[0]), R(0));
+                        S.best = SC::round(SC::get(n[0]));
+                        S.since = 0;
+                        S.idone = 0;
+                        S.itc = 0;
+                        const double need = 0.5 * A.tol * sqrt(S.bn2 / fmax(S.rn2, 1e-300));
+                        const double it = fmax(A.inner_tol, need);
+                        S.itol2 = it * it;
+                    }))
+                    return;
+            }
+
+            if constexpr (METHOD == SOLVER_SERIES) {
+                // ---- p <- (r + k2 H_eo H_oe p) / diag from p = r, the residual
+                // reduced every second iteration (as in k_solve)
+                const T k2 = (T)A.k2, dinv = (T)(1.0 / A.diag);
+                for (;;) {
+                    const bool chk = (S.itc & 1) || S.itc + 1 >= A.max_inner || S.it + 1 >= A.max_iter;
+                    Acc<T> q[1] = {Acc<T>::zero()};
+#pragma unroll 1
+                    for (int par = 1; par >= 0; --par) {
+                        const W* in = par ? V_(p) : V_(tmp);
+                        FOR_GROUPS
+                        {
+                            Spinor<T> acc;
+                            cx<T> o[NC];
+                            hop_part<P, LPS>(A.g, A.mode, par, i, d, in, UP, acc);
+                            xc.combine(NW, acc, o);
+                            if (xc.fin() && on) {
+                                if (par) {
+                                    store_part<NC>(V_(tmp) + at, d, o);
+                                } else {
+                                    cx<T> pp[NC], rr[NC];
+                                    load_part<NC>(V_(p) + at, d, pp);
+                                    load_part<NC>(V_(r) + at, d, rr);
+#pragma unroll
+                                    for (int k = 0; k < NC; ++k) {
+                                        o[k] = dinv * (rr[k] + k2 * o[k]);
+                                        pp[k] = o[k] - pp[k];
+                                    }
+                                    store_part<NC>(V_(p) + at, d, o);
+                                    if (chk) q[0].add(pnorm<NC>(pp));
+                                }
+                            }
+                        }
+                        if (par) SYNC_OR_RETURN;
+                    }
+                    if (!chk) {
+                        SYNC_OR_RETURN;
+                        if (tid == 0) {
+                            S.it += 1;
+                            S.itc += 1;
+                        }
+                        __syncthreads();
+                        continue;
+                    }
+                    if (!group_reduce<NW, 1>(A, G, q, [&](const Acc<T>(&n)[1]) {
+                            S.it += 1;
+                            S.itc += 1;
+                            const double res2 = A.diag * A.diag * (double)SC::round(SC::get(n[0]));
+                            if (!(res2 > S.itol2) || S.itc >= A.max_inner || S.it >= A.max_iter) S.idone = 1;
+                            // a series that grows cannot converge: reported as not converged
+                            if (!isfinite(res2) || (S.itc >= 16 && res2 > 1e6)) {
+                                S.idone = 1;
+                                S.it = A.max_iter;
+                            }
+                        }))
+                        return;
+                    if (S.idone) break;
+                }
+            } else {
+                // ---- BiCGstab, six barriers an iteration, two of them reducing:
+                //   0  tmp = H_oe p        1  v = A p, <rh, v> -> alpha      s = r - alpha v
+                //   2  tmp = H_oe s        3  t = A s and the sums of omega, beta
+                //   e += alpha p + omega s, r = s - omega t, p = r + beta (p - omega v)
+                // <rh, r> and |r|^2 of the new residual follow from the sums of step
+                // 3, so beta is known before r is formed.  One copy of the
+                // hopping code serves all four sweeps: it has to fit the
+                // instruction cache.
+                const T k2 = (T)A.k2, dg = (T)A.diag;
+                bool stop = false;
+                for (;;) {
+#pragma unroll 1
+                    for (int ph = 0; ph < 4; ++ph) {
+                        const W* in = ph == 0 ? V_(p) : ph == 2 ? V_(r) : V_(tmp);
+                        // the thread's sums wait in shared memory: sixteen registers less in the hops
+                        bool some = false;
+                        FOR_GROUPS
+                        {
+                            Spinor<T> acc;
+                            cx<T> o[NC];
+                            hop_part<P, LPS>(A.g, A.mode, 1 - (ph & 1), i, d, in, UP, acc);
+                            xc.combine(NW, acc, o);
+                            if (xc.fin() && on) {
+                                if (!(ph & 1)) {
+                                    store_part<NC>(V_(tmp) + at, d, o);
+                                } else {
+                                    cx<T> y[NC], z[NC];
+                                    load_part<NC>((ph == 1 ? V_(p) : V_(r)) + at, d, y);
+                                    load_part<NC>(V_(rh) + at, d, z);
+#pragma unroll
+                                    for (int k = 0; k < NC; ++k) o[k] = dg * y[k] - k2 * o[k];
+                                    store_part<NC>((ph == 1 ? V_(v) : V_(t)) + at, d, o);
+                                    T n[8];
+                                    pdot<NC>(z, o, n[0], n[1]);
+                                    if (ph == 3) {
+                                        pdot<NC>(z, y, n[2], n[3]);
+                                        pdot<NC>(o, y, n[4], n[5]);
+                                        n[6] = pnorm<NC>(o);
+                                        n[7] = pnorm<NC>(y);
+                                    }
+#pragma unroll
+                                    for (int k = 0; k < 8; ++k)
+                                        if (k < 2 || ph == 3) {
+                                            Acc<T> s = Acc<T>::zero();
+                                            if (some) s = sums[k][tid];
+                                            s.add(n[k]);
+                                            sums[k][tid] = s;
+                                        }
+                                    some = true;
+                                }
+                            }
+                        }
+                        Acc<T> q[8];
+#pragma unroll
+                        for (int k = 0; k < 8; ++k) {
+                            q[k] = Acc<T>::zero();
+                            if (some && (k < 2 || ph == 3)) q[k] = sums[k][tid];
+                        }
+                        if (!(ph & 1)) {
+                            SYNC_OR_RETURN;
+                        } else if (ph == 1) {
+                            Acc<T> q2[4] = {q[0], q[1], Acc<T>::zero(), Acc<T>::zero()};
+                            if (!group_reduce<NW, 4>(A, G, q2, [&](const Acc<T>(&n)[4]) {
+                                    const cx<R> dn = mk(SC::get(n[0]), SC::get(n[1]));
+                                    const cx<T> d0 = sround<T>(dn), al = sround<T>(SC::div(S.rho, dn));
+                                    S.d = dn;
+                                    if (!fin2(al) || (d0.re == T(0) && d0.im == T(0))) S.idone = 1;
+                                    else S.alpha = al;
+                                }))
+                                return;
+                            if (S.idone) {  // the sums gave no step
+                                stop = true;
+                                break;
+                            }
+                            const cx<T> mal = -S.alpha;
+                            for_words<3, NWORD, NW>(
+                                WORDS, [&](int i, int k) { return W2<W>{V_(r)[TW(i, k)], V_(v)[TW(i, k)]}; },
+                                [&](int i, int k, W2<W> w) { V_(r)[TW(i, k)] = waxpy(mal, w.y, w.x); });
+                            SYNC_OR_RETURN;
+                        } else {
+                            if (!group_reduce<NW, 8>(A, G, q, [&](const Acc<T>(&n)[8]) {
+                                    const cx<R> rt = mk(SC::get(n[0]), SC::get(n[1])), rs = mk(SC::get(n[2]), SC::get(n[3]));
+                                    const cx<R> ts = mk(SC::get(n[4]), SC::get(n[5]));
+                                    const R tt = SC::get(n[6]), ss = SC::get(n[7]);
+                                    cx<T> om = sround<T>(SC::div(ts, mk(tt, R(0))));
+                                    if (!(SC::round(tt) > T(0)) || !fin2(om)) {
+                                        om = mk(T(0), T(0));
+                                        S.idone = 1;  // keep alpha p, stop afterwards
+                                    }
+                                    S.omega = om;
+                                    S.it += 1;
+                                    S.itc += 1;
+                                    const cx<R> omr = mk(from_round<R>(om.re), from_round<R>(om.im));
+                                    const cx<R> rn = rs - omr * rt;
+                                    // |s - omega t|^2
+                                    const R two = from_round<R>(T(2));
+                                    const R rr = ss - two * (omr.re * ts.re + omr.im * ts.im) +
+                                                 (omr.re * omr.re + omr.im * omr.im) * tt;
+                                    const T rf = SC::round(rr);
+                                    // far above its start (1) the recurrence has diverged: keep the
+                                    // correction so far, the outer cycle recomputes the residual
+                                    if (S.itc >= A.max_inner || S.it >= A.max_iter || !((double)rf > S.itol2) ||
+                                        !fin2(sround<T>(rn)) || rf > T(1e8))
+                                        S.idone = 1;
+                                    // a residual that has stalled: restarted from the true one
+                                    if (rf < S.best) {
+                                        S.best = rf;
+                                        S.since = 0;
+                                    } else if (++S.since >= STALL) {
+                                        S.idone = 1;
+                                    }
+                                    if (!S.idone) {
+                                        // beta = (rn / rho) (alpha / omega) with alpha = rho / d
+                                        const cx<T> be = sround<T>(SC::div(rn, S.d * omr));
+                                        if (!fin2(be)) S.idone = 1;
+                                        S.beta = be;
+                                        S.rho = rn;
+                                    }
+                                }))
+                                return;
+                        }
+                    }
+                    if (stop) break;
+                    {
+                        const cx<T> al = S.alpha, om = S.omega, be = S.beta;
+                        const bool more = !S.idone;
+                        constexpr int B = P == PREC32 ? 3 : 2;
+                        for_words<B, NWORD, NW>(
+                            WORDS,
+                            [&](int i, int k) {
+                                const size_t a = TW(i, k);
+                                return W5<W>{V_(r)[a], V_(t)[a], V_(v)[a], V_(p)[a], V_(e)[a]};
+                            },
+                            [&](int i, int k, W5<W> w) {
+                                const size_t a = TW(i, k);
+                                V_(e)[a] = waxpy(om, w.s, waxpy(al, w.p, w.e));
+                                if (more) {
+                                    const W rr = waxpy(-om, w.t, w.s);
+                                    V_(r)[a] = rr;
+                                    V_(p)[a] = waxpy(be, waxpy(-om, w.v, w.p), rr);
+                                }
+                            });
+                    }
+                    if (S.idone) break;
+                    SYNC_OR_RETURN;
+                }
+                SYNC_OR_RETURN;
+            }
+
+            // ---- x += |r64| e
+            {
+                const double sc = sqrt(S.rn2);
+                const W* ev = METHOD == SOLVER_SERIES ? V_(p) : V_(e);
+                for_words<2, 12, NW>(
+                    WORDS,
+                    [&](int i, int c) {
+                        W2<double2> r;
+                        r.x = xx[DW(i, c)];
+                        if constexpr (P == PREC32) {
+                            const float2 w = ((const float2*)ev)[TW(i, c >> 1) * 2 + (c & 1)];
+                            r.y = make_double2(w.x, w.y);
+                        } else {
+                            r.y = ev[TW(i, c)];
+                        }
+                        return r;
+                    },
+                    [&](int i, int c, W2<double2> w) {
+                        const size_t a = DW(i, c);
+                        const double re = w.x.x + sc * w.y.x, im = w.x.y + sc * w.y.y;
+                        xx[a] = make_double2(re, im);
+                        if (P == PREC32) store_split((float4*)xs.v + a, re, im);
+                    });
+            }
+            SYNC_OR_RETURN;
+            fresh = true;
+        }
+
+        if (leader) {
+            A.iters[sys] = S.it;
+            A.resid[sys] = S.bn2 > 0.0 ? sqrt(S.rn2 / S.bn2) : 0.0;
+            if (sys == 0) *A.outer_out = outer;
+            const int err = final_flag == F_NAN ? LQCD_ERR_NAN : final_flag == F_MAXIT ? LQCD_ERR_NOCONVERGE : 0;
+            if (err) {
+                atomicCAS(A.status, 0, err);
+                atomicCAS(A.sticky, 0, err);
+            }
+            atomicAdd(A.acc, (unsigned long long)S.it);
+            atomicAdd(A.acc + (METHOD == SOLVER_SERIES ? 3 : 1), (unsigned long long)S.it * (unsigned long long)A.nsite);
+            atomicAdd(A.acc + 2, (unsigned long long)outer * (unsigned long long)A.nsite);
+        }
+        __syncthreads();  // S belongs to the next system from here on
+    }
+#undef V_
+#undef SYNC_OR_RETURN
+#undef FOR_GROUPS
+#undef FOR_ITEMS
+#undef WORDS
+#undef TW
+#undef DW
+}
+
+}  // namespace
+
+// ---------------------------------------------------------------------------
+// host side
+// ---------------------------------------------------------------------------
+namespace {
+
+struct Variant {
+    const void* fn[2];  // BiCGstab, series
+    int prec, lps, bs, smem;
+};
+
+template <int P, int LPS, int BS, int MINB>
+constexpr Variant variant()
+{
+    return Variant{{(const void*)k_split<P, LPS, BS, MINB, SOLVER_BICGSTAB>,
+                    (const void*)k_split<P, LPS, BS, MINB, SOLVER_SERIES>},
+                   P, LPS, BS, split_smem<P, LPS, BS>()};
+}
+
+enum { V_F64 = 0, V_8, V_4, V_2, V_1, V_1W };
+const Variant variants[SPLIT_NVAR] = {variant<PREC64, 8, 256, 1>(), variant<PREC32, 8, 256, 2>(),
+                                      variant<PREC32, 4, 256, 2>(), variant<PREC32, 2, 256, 2>(),
+                                      variant<PREC32, 1, 256, 2>(), variant<PREC32, 1, 512, 1>()};
+
+// The kernel for `groups` groups of 32 sites over all systems.  Double
+// precision is bound by the FP64 pipe, which eight warps fill.  Single
+// precision, measured (ms per solve, LPS 8 / 4 / 2 / 1): 41 groups 2.23 / 2.36 /
+// 2.71 / 3.25, 128 groups 2.23 / 2.26 / 2.55 / 3.24, 300 groups 2.73 / 2.41 /
+// 2.50 / 3.17, 648 groups 16.3 / 14.2 / 13.3 / 13.1, 1024 groups 16.2 / 13.9 /
+// 12.0 / 11.9: LPS 8 while every group has an SM of its own, then 4 and 2 while
+// the groups still fit the SMs side by side.  From 2432 groups on (more than
+// two CTAs of eight groups per SM) one CTA of 512 threads per SM halves the
+// barrier's arrivals (6912 groups 66.3 against 67.6, 32768 groups 420 / 431).
+int pick(int prec, int groups, int num_sms)
+{
+    if (prec == PREC64) return V_F64;
+    if (8 * groups <= 7 * num_sms) return V_8;
+    if (groups <= 2 * num_sms) return V_4;
+    if (groups <= 4 * num_sms) return V_2;
+    return groups <= 16 * num_sms ? V_1 : V_1W;
+}
+
+}  // namespace
+
+cudaError_t split_init(int num_sms, int occ[SPLIT_NVAR][2], int* gmax)
+{
+    *gmax = 0;
+    for (int k = 0; k < SPLIT_NVAR; ++k)
+        for (int m = 0; m < 2; ++m) {
+            const Variant& v = variants[k];
+            cudaError_t e = cudaFuncSetAttribute(v.fn[m], cudaFuncAttributeMaxDynamicSharedMemorySize, v.smem);
+            if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[k][m], v.fn[m], v.bs, v.smem);
+            if (e != cudaSuccess) return e;
+            if (occ[k][m] < 1) return cudaErrorLaunchOutOfResources;
+            *gmax = std::max(*gmax, occ[k][m] * num_sms);
+        }
+    return cudaSuccess;
+}
+
+SplitPlan split_plan(SolveArgs& A, int prec, int method, int spt, int num_sms, const int occ[SPLIT_NVAR][2])
+{
+    const int G = (A.nsite + 31) / 32;
+    const int k = pick(prec, G * A.nsys, num_sms), m = method == SOLVER_SERIES ? 1 : 0;
+    const Variant& v = variants[k];
+    const int SG = v.bs / 32 / v.lps;  // groups a CTA holds side by side
+    const int want = spt <= 0 ? G : (G + SG * spt - 1) / (SG * spt);
+    A.ngrp = A.nsys;
+    A.cps = std::max(1, std::min(occ[k][m] * num_sms / A.ngrp, want));
+    const int gpc = (G + A.cps - 1) / A.cps;
+    A.cps = (G + gpc - 1) / gpc;
+    A.chunk = gpc * 32;
+    // tiles of 16 groups where the CTAs make several passes (64x32^3: 420
+    // against 454 ms) and whole planes are whole groups; a single pass is no
+    // faster for it (32x16^3: 23.0 against 22.3)
+    A.tiled = 0;
+    const Geo& g = A.g;
+    const int plane = g.L[2] * g.L[3] / 2;
+    if (gpc > SG && g.lg[0] && plane >= 32) {
+        int left = 4;
+        auto take = [&](int n, int most) {
+            int l = 0;
+            while (l < most && l < left && n % (2 << l) == 0) ++l;
+            left -= l;
+            return l;
+        };
+        A.lt[0] = take(A.nsite / (g.L[1] * plane), 2);
+        A.lt[1] = take(g.L[1], 2);
+        A.lt[2] = take(plane / 32, 4);
+        A.nt[0] = g.lg[1] - A.lt[1];
+        A.nt[1] = g.lg[2] + g.lg[3] - 6 - A.lt[2];
+        A.tiled = 1;
+    }
+    return SplitPlan{v.fn[m], A.cps * A.ngrp, v.bs, v.smem};
+}
