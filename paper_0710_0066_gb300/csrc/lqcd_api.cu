@@ -50,6 +50,17 @@ SpinorF none()
     return f;
 }
 
+// parity block of work field k as a field of a low storage precision (room
+// for a double block)
+SpinorF low_view(lqcd_ctx* h, int k, int prec, int par)
+{
+    SpinorF f;
+    f.v = (char*)fld(h, k) + (size_t)par * 12 * h->g.Vh * sizeof(double2);
+    f.N = h->g.Vh;
+    f.nrm = prec == PREC16 ? (float*)((uint4*)f.v + (size_t)3 * h->g.Vh) : nullptr;
+    return f;
+}
+
 // full-lattice out = a x + c H_mode in on the output slabs of `colour`
 int hop_full(lqcd_ctx* h, int mode, int dag, int colour, double2* out, const double2* in, double a,
              const double2* x, double c)
@@ -1085,37 +1096,26 @@ int lqcd_dslash_eo(lqcd_t h, double* out, const double* in, double kappa, int pa
     NEED(op == LQCD_OP_HOP || (op == LQCD_OP_MHAT && parity == 0), "op must be HOP, or MHAT with parity 0");
     NEED(prec_ok(precision), "bad precision");
     const int Vh = h->g.Vh;
-    double2 *A = fld(h, F_A), *B = fld(h, F_B);
+    double2* A = fld(h, F_A);
     const int pin = op == LQCD_OP_HOP ? 1 - parity : 0;
-    LQ_TRY(pack_spinor(h, A, in, pin, 1));
-    // low-precision work fields live in F_C / F_D (same byte size as double)
-    SpinorF src = sp64(A, pin, Vh), res = sp64(B, parity, Vh);
+    double2* abi = (double2*)out;
     if (precision != LQCD_PREC_F64) {
-        auto lowview = [&](double2* buf, int par) {
-            SpinorF f;
-            f.v = (char*)buf + (size_t)par * 12 * Vh * sizeof(double2);
-            f.N = Vh;
-            f.nrm = precision == PREC16 ? (float*)((uint4*)f.v + (size_t)3 * Vh) : nullptr;
-            return f;
-        };
-        SpinorF ls = lowview(fld(h, F_C), pin), lr = lowview(fld(h, F_D), parity);
-        LQ_TRY(convert_spinor(h, ls, precision, src, PREC64, Vh));
-        if (op == LQCD_OP_HOP) {
-            LQ_TRY(hop_sweep(h, precision, MODE_ALL, dagger, parity, -1, lr, ls, 0.0, none(), 1.0));
-        } else {
-            SpinorF lt = lowview(fld(h, F_E), 1);
-            LQ_TRY(hop_sweep(h, precision, MODE_ALL, dagger, 1, -1, lt, ls, 0.0, none(), 1.0));
-            LQ_TRY(hop_sweep(h, precision, MODE_ALL, dagger, 0, -1, lr, lt, 1.0, ls, -kappa * kappa));
-        }
-        LQ_TRY(convert_spinor(h, res, PREC64, lr, precision, Vh));
-    } else if (op == LQCD_OP_HOP) {
-        LQ_TRY(hop_sweep(h, PREC64, MODE_ALL, dagger, parity, -1, res, src, 0.0, none(), 1.0));
-    } else {
-        SpinorF tt = sp64(fld(h, F_C), 1, Vh);
-        LQ_TRY(hop_sweep(h, PREC64, MODE_ALL, dagger, 1, -1, tt, src, 0.0, none(), 1.0));
-        LQ_TRY(hop_sweep(h, PREC64, MODE_ALL, dagger, 0, -1, res, tt, 1.0, src, -kappa * kappa));
+        // low-precision work fields live in F_C / F_D (same byte size as double)
+        SpinorF ls = low_view(h, F_C, precision, pin);
+        LQ_TRY(pack_spinor_low(h, ls, precision, in));
+        if (op == LQCD_OP_HOP)
+            return hop_sweep(h, precision, MODE_ALL, dagger, parity, -1, none(), ls, 0.0, none(), 1.0, abi);
+        SpinorF lt = low_view(h, F_E, precision, 1);
+        LQ_TRY(hop_sweep(h, precision, MODE_ALL, dagger, 1, -1, lt, ls, 0.0, none(), 1.0));
+        return hop_sweep(h, precision, MODE_ALL, dagger, 0, -1, none(), lt, 1.0, ls, -kappa * kappa, abi);
     }
-    return unpack_spinor(h, out, B, parity, 1);
+    LQ_TRY(pack_spinor(h, A, in, pin, 1));
+    const SpinorF src = sp64(A, pin, Vh);
+    if (op == LQCD_OP_HOP)
+        return hop_sweep(h, PREC64, MODE_ALL, dagger, parity, -1, none(), src, 0.0, none(), 1.0, abi);
+    SpinorF tt = sp64(fld(h, F_C), 1, Vh);
+    LQ_TRY(hop_sweep(h, PREC64, MODE_ALL, dagger, 1, -1, tt, src, 0.0, none(), 1.0));
+    return hop_sweep(h, PREC64, MODE_ALL, dagger, 0, -1, none(), tt, 1.0, src, -kappa * kappa, abi);
 }
 
 }  // extern "C"
@@ -1125,27 +1125,19 @@ static int block_dslash_impl(lqcd_t h, double* out, const double* in, double kap
                              int precision)
 {
     const int Vh = h->g.Vh;
-    double2 *A = fld(h, F_A), *B = fld(h, F_B);
-    LQ_TRY(pack_spinor(h, A, in, 0, 2));
-    if (precision == LQCD_PREC_F64) {
-        LQ_TRY(hop_full(h, MODE_INTRA, dagger, colour, B, A, 1.0, A, -kappa));
-    } else {
-        auto lowview = [&](double2* buf, int par) {
-            SpinorF f;
-            f.v = (char*)buf + (size_t)par * 12 * Vh * sizeof(double2);
-            f.N = Vh;
-            f.nrm = precision == PREC16 ? (float*)((uint4*)f.v + (size_t)3 * Vh) : nullptr;
-            return f;
-        };
-        for (int p = 0; p < 2; ++p) LQ_TRY(convert_spinor(h, lowview(fld(h, F_C), p), precision, sp64(A, p, Vh), PREC64, Vh));
-        for (int p = 0; p < 2; ++p)
-            LQ_TRY(hop_sweep(h, precision, MODE_INTRA, dagger, p, colour, lowview(fld(h, F_D), p),
-                             lowview(fld(h, F_C), 1 - p), 1.0, lowview(fld(h, F_C), p), -kappa));
-        LQ_CUDA(h, cudaMemsetAsync(B, 0, sizeof(double2) * 24 * (size_t)Vh, h->stream));
-        for (int p = 0; p < 2; ++p) LQ_TRY(convert_spinor(h, sp64(B, p, Vh), PREC64, lowview(fld(h, F_D), p), precision, Vh));
-        if (colour >= 0) LQ_TRY(keep_colour(h, B, colour));
+    if (precision == LQCD_PREC_F64) LQ_TRY(pack_spinor(h, fld(h, F_A), in, 0, 2));
+    for (int p = 0; p < 2 && precision != LQCD_PREC_F64; ++p)
+        LQ_TRY(pack_spinor_low(h, low_view(h, F_C, precision, p), precision, in + (size_t)p * 24 * Vh));
+    for (int p = 0; p < 2; ++p) {
+        double2* abi = (double2*)out + (size_t)p * 12 * Vh;
+        if (precision == LQCD_PREC_F64)
+            LQ_TRY(hop_sweep(h, PREC64, MODE_INTRA, dagger, p, colour, none(), sp64(fld(h, F_A), 1 - p, Vh), 1.0,
+                             sp64(fld(h, F_A), p, Vh), -kappa, abi));
+        else
+            LQ_TRY(hop_sweep(h, precision, MODE_INTRA, dagger, p, colour, none(), low_view(h, F_C, precision, 1 - p),
+                             1.0, low_view(h, F_C, precision, p), -kappa, abi));
     }
-    return unpack_spinor(h, out, B, 0, 2);
+    return LQCD_OK;
 }
 
 static int block_solve_impl(lqcd_t h, double* x, const double* b, double kappa, int colour, int dagger,
@@ -1576,15 +1568,8 @@ int lqcd_autotune(lqcd_t h, int what, double kappa)
         for (int prec = 0; prec < NPREC && st == LQCD_OK; ++prec) {
             SpinorF in = sp64(A, 1, Vh), out = sp64(B, 0, Vh);
             if (prec != PREC64) {
-                auto lowview = [&](double2* buf, int par) {
-                    SpinorF f;
-                    f.v = (char*)buf + (size_t)par * 12 * Vh * sizeof(double2);
-                    f.N = Vh;
-                    f.nrm = prec == PREC16 ? (float*)((uint4*)f.v + (size_t)3 * Vh) : nullptr;
-                    return f;
-                };
-                in = lowview(fld(h, F_C), 1);
-                out = lowview(fld(h, F_D), 0);
+                in = low_view(h, F_C, prec, 1);
+                out = low_view(h, F_D, prec, 0);
                 st = convert_spinor(h, in, prec, sp64(A, 1, Vh), PREC64, Vh);
             }
             // candidates interleaved over four rounds, the minimum per

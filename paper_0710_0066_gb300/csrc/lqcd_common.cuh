@@ -156,6 +156,36 @@ LQ_HD void complete_row2(Su3<T>& u)
     u.m[2][2] = conjx(u.m[0][0] * u.m[1][1] - u.m[0][1] * u.m[1][0]);
 }
 
+// a b + c and a^* b + c as chains of fused multiply-adds.  The FP64 kernels
+// are bound by the number of FP64 instructions, and the compiler does not
+// join the additions between complex products with them: 12 instructions per
+// entry of a 3-vector product instead of 16.
+LQ_HD cx<double> cfma(cx<double> a, cx<double> b, cx<double> c)
+{
+    return {fma(-a.im, b.im, fma(a.re, b.re, c.re)), fma(a.im, b.re, fma(a.re, b.im, c.im))};
+}
+LQ_HD cx<double> cjfma(cx<double> a, cx<double> b, cx<double> c)
+{
+    return {fma(a.im, b.im, fma(a.re, b.re, c.re)), fma(-a.im, b.re, fma(a.re, b.im, c.im))};
+}
+// a0 b0 + a1 b1 + a2 b2 (first factors conjugated: cjdot3); the other types
+// keep the plain form, whose rounding their results are known by
+template <class T>
+LQ_HD cx<T> cdot3(cx<T> a0, cx<T> b0, cx<T> a1, cx<T> b1, cx<T> a2, cx<T> b2) { return a0 * b0 + a1 * b1 + a2 * b2; }
+template <class T>
+LQ_HD cx<T> cjdot3(cx<T> a0, cx<T> b0, cx<T> a1, cx<T> b1, cx<T> a2, cx<T> b2)
+{
+    return cjmul(a0, b0) + cjmul(a1, b1) + cjmul(a2, b2);
+}
+LQ_HD cx<double> cdot3(cx<double> a0, cx<double> b0, cx<double> a1, cx<double> b1, cx<double> a2, cx<double> b2)
+{
+    return cfma(a2, b2, cfma(a1, b1, cx<double>{fma(-a0.im, b0.im, a0.re * b0.re), fma(a0.im, b0.re, a0.re * b0.im)}));
+}
+LQ_HD cx<double> cjdot3(cx<double> a0, cx<double> b0, cx<double> a1, cx<double> b1, cx<double> a2, cx<double> b2)
+{
+    return cjfma(a2, b2, cjfma(a1, b1, cx<double>{fma(a0.im, b0.im, a0.re * b0.re), fma(-a0.im, b0.re, a0.re * b0.im)}));
+}
+
 // w = u v  /  w = u^dag v  on the two spin rows of a half spinor
 template <class T>
 LQ_HD void su3_mul_half(const Su3<T>& u, const HalfSp<T>& h, HalfSp<T>& w)
@@ -164,7 +194,7 @@ LQ_HD void su3_mul_half(const Su3<T>& u, const HalfSp<T>& h, HalfSp<T>& w)
     for (int s = 0; s < 2; ++s)
 #pragma unroll
         for (int i = 0; i < 3; ++i)
-            w.c[s][i] = u.m[i][0] * h.c[s][0] + u.m[i][1] * h.c[s][1] + u.m[i][2] * h.c[s][2];
+            w.c[s][i] = cdot3(u.m[i][0], h.c[s][0], u.m[i][1], h.c[s][1], u.m[i][2], h.c[s][2]);
 }
 template <class T>
 LQ_HD void su3_dagmul_half(const Su3<T>& u, const HalfSp<T>& h, HalfSp<T>& w)
@@ -173,8 +203,7 @@ LQ_HD void su3_dagmul_half(const Su3<T>& u, const HalfSp<T>& h, HalfSp<T>& w)
     for (int s = 0; s < 2; ++s)
 #pragma unroll
         for (int i = 0; i < 3; ++i)
-            w.c[s][i] = cjmul(u.m[0][i], h.c[s][0]) + cjmul(u.m[1][i], h.c[s][1]) +
-                        cjmul(u.m[2][i], h.c[s][2]);
+            w.c[s][i] = cjdot3(u.m[0][i], h.c[s][0], u.m[1][i], h.c[s][1], u.m[2][i], h.c[s][2]);
 }
 
 // ---------------------------------------------------------------------------
@@ -512,6 +541,29 @@ template <int P>
 __device__ __forceinline__ void store_spinor(const SpinorF& f, int i, const Spinor<typename Real<P>::T>& s)
 {
     SpIO<P, true>::store(f, i, s);
+}
+
+// a spinor as storing it in half storage P and reading it back leaves it
+template <int P>
+__device__ __forceinline__ void round_spinor(Spinor<float>& s)
+{
+    static_assert(P == PREC16 || P == PRECBF, "half storage");
+    float mx = 0.f;
+#pragma unroll
+    for (int c = 0; c < 12; ++c)
+        mx = fmaxf(mx, fmaxf(fabsf(s.c[c / 3][c % 3].re), fabsf(s.c[c / 3][c % 3].im)));
+    const float inv = mx > 0.f ? 1.0f / mx : 0.f;
+#pragma unroll
+    for (int c = 0; c < 12; ++c) {
+        cx<float>& v = s.c[c / 3][c % 3];
+        if (P == PREC16) {
+            const float2 f = __half22float2(__floats2half2_rn(v.re * inv, v.im * inv));
+            v = mk(f.x * mx, f.y * mx);
+        } else {
+            const float2 f = __bfloat1622float2(__floats2bfloat162_rn(v.re, v.im));
+            v = mk(f.x, f.y);
+        }
+    }
 }
 
 // gauge links ----------------------------------------------------------------
@@ -1049,6 +1101,8 @@ int pack_spinor(lqcd_ctx* h, double2* dst, const double* abi, int parity_first, 
 int unpack_spinor(lqcd_ctx* h, double* abi, const double2* src, int parity_first, int nparity);
 int pack_gauge(lqcd_ctx* h, const double* abi);
 int unpack_gauge(lqcd_ctx* h, double* abi);
+// one parity of a C-ABI field into storage precision prec (not double)
+int pack_spinor_low(lqcd_ctx* h, SpinorF dst, int prec, const double* abi);
 int convert_spinor(lqcd_ctx* h, SpinorF dst, int dprec, SpinorF src, int sprec, int n);
 int index_maps(lqcd_ctx* h, int32_t* maps);
 // boundary space of the active geometry; nface = 2: both faces of every
@@ -1079,8 +1133,10 @@ int read_scalars(lqcd_ctx* h, int n, double* host);
 // dslash.cu
 // out(p_out) = a * x(p_out) + c * H_{p_out,1-p_out} in(1-p_out) on the output
 // sites of slabs with the given colour (-1: all); x may be null (a ignored)
+// abi: the result goes to this one-parity field of the C-ABI (double, site by
+// site) instead of out, with zeros on the slabs of the other colour
 int hop_sweep(lqcd_ctx* h, int prec, int mode, int dag, int pout, int colour, SpinorF out,
-              SpinorF in, double a, SpinorF x, double c);
+              SpinorF in, double a, SpinorF x, double c, double2* abi = nullptr);
 
 // solver.cu
 int solver_init(lqcd_ctx* h);

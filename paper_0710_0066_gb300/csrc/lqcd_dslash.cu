@@ -115,46 +115,120 @@ __device__ __forceinline__ void hop_site_h16(const Geo& g, int mode, int dag, in
     }
 }
 
+// The warp's 32 results to the C-ABI layout, double[site][4][3][2]: each
+// lane's 24 numbers pass through shared memory (rows of 13: no bank conflict
+// beyond the width) so that the stores run along the sites.  Stored straight
+// from the lanes, 192 bytes apart, every 32-byte sector is written in two
+// halves.  S: the type a result fits exactly; `i`, `on` per lane.
+// An operator call is bound by HBM; its C-ABI field alone is 192 bytes a site
+// each way, so passes over it are what counts: packing to double, converting,
+// sweeping, converting back, unpacking and the clearing of a result that is
+// written in full moved 1900 bytes a site in single precision, packing
+// straight to the sweep's storage and this store 864.  A call at 64x32^3 in
+// single precision 506 -> 178 us, at 32x24^3 in half precision 117 -> 44 us.
+template <class S>
+struct Pair {
+    S re, im;
+};
+template <class S, int NC, class T>
+__device__ __forceinline__ void abi_store(Pair<S>* sh, double2* abi, int i, bool on, const Spinor<T>& acc)
+{
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int c0 = 0; c0 < 12; c0 += NC) {
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < NC; ++k) {
+            const cx<T> v = acc.c[(c0 + k) / 3][(c0 + k) % 3];
+            sh[lane * (NC + 1) + k] = Pair<S>{(S)v.re, (S)v.im};
+        }
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < NC; ++k) {
+            const int e = k * 32 + lane, site = e / NC, c = e % NC;
+            const int j = __shfl_sync(0xffffffffu, i, site);
+            const bool ok = __shfl_sync(0xffffffffu, (int)on, site) != 0;
+            const Pair<S> v = sh[site * (NC + 1) + c];
+            if (ok) abi[(size_t)j * 12 + c0 + c] = make_double2((double)v.re, (double)v.im);
+        }
+    }
+}
+
+// complex numbers of a site that pass through shared memory at a time, and
+// the shared memory of a block
 template <int P>
+constexpr int abi_chunk()
+{
+    return P == PREC64 ? 6 : 12;
+}
+template <int P>
+constexpr int abi_smem(int bs)
+{
+    return bs * (abi_chunk<P>() + 1) * 2 * (int)sizeof(typename Real<P>::T);
+}
+
+template <int P, bool ABI>
 __device__ __forceinline__ void hop_body(Geo g, int mode, int dag, int pout, int colour, SpinorF out, SpinorF in,
-                                         GaugeF U, double a, SpinorF x, double c, int nsites)
+                                         GaugeF U, double a, SpinorF x, double c, int nsites, double2* abi)
 {
     typedef typename Real<P>::T T;
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= nsites) return;
-    int i = t;
+    const bool on = t < nsites;
+    if (!ABI && !on) return;
+    int i = on ? t : nsites - 1;
+    bool mine = true;
     if (colour >= 0) {
-        const int k = t / g.Sh;
-        i = (colour + 2 * k) * g.Sh + (t - k * g.Sh);
+        if (ABI) {  // every site, zeros on the other colour's slabs
+            mine = ((i / g.Sh) & 1) == colour;
+        } else {
+            const int k = t / g.Sh;
+            i = (colour + 2 * k) * g.Sh + (t - k * g.Sh);
+        }
     }
     Spinor<T> acc;
-    if constexpr (P == PREC16)
-        hop_site_h16(g, mode, dag, pout, i, in, U, acc);
-    else
-        hop_site<P>(g, mode, dag, pout, i, in, U, acc);
-    const T cc = (T)c;
-    if (x.v) {
-        Spinor<T> xs;
-        load_spinor<P>(x, i, xs);
-        const T aa = (T)a;
+    if (mine) {
+        if constexpr (P == PREC16)
+            hop_site_h16(g, mode, dag, pout, i, in, U, acc);
+        else
+            hop_site<P>(g, mode, dag, pout, i, in, U, acc);
+        const T cc = (T)c;
+        if (x.v) {
+            Spinor<T> xs;
+            load_spinor<P>(x, i, xs);
+            const T aa = (T)a;
 #pragma unroll
-        for (int s = 0; s < 4; ++s)
+            for (int s = 0; s < 4; ++s)
 #pragma unroll
-            for (int q = 0; q < 3; ++q) acc.c[s][q] = aa * xs.c[s][q] + cc * acc.c[s][q];
+                for (int q = 0; q < 3; ++q) acc.c[s][q] = aa * xs.c[s][q] + cc * acc.c[s][q];
+        } else {
+#pragma unroll
+            for (int s = 0; s < 4; ++s)
+#pragma unroll
+                for (int q = 0; q < 3; ++q) acc.c[s][q] = cc * acc.c[s][q];
+        }
     } else {
 #pragma unroll
         for (int s = 0; s < 4; ++s)
 #pragma unroll
-            for (int q = 0; q < 3; ++q) acc.c[s][q] = cc * acc.c[s][q];
+            for (int q = 0; q < 3; ++q) acc.c[s][q] = mk(T(0), T(0));
     }
-    store_spinor<P>(out, i, acc);
+    if constexpr (ABI) {
+        // half storage rounds the result to the storage format: through it
+        extern __shared__ __align__(16) unsigned char hop_dyn[];
+        constexpr int NC = abi_chunk<P>();
+        if constexpr (P == PREC16 || P == PRECBF) round_spinor<P>(acc);
+        abi_store<T, NC>((Pair<T>*)hop_dyn + (threadIdx.x >> 5) * 32 * (NC + 1), abi, i, on, acc);
+    } else {
+        store_spinor<P>(out, i, acc);
+    }
 }
 
-template <int P>
+template <int P, bool ABI>
 __global__ void __launch_bounds__(HOP_BS_MAX) k_hop(Geo g, int mode, int dag, int pout, int colour, SpinorF out,
-                                               SpinorF in, GaugeF U, double a, SpinorF x, double c, int nsites)
+                                               SpinorF in, GaugeF U, double a, SpinorF x, double c, int nsites,
+                                               double2* abi)
 {
-    hop_body<P>(g, mode, dag, pout, colour, out, in, U, a, x, c, nsites);
+    hop_body<P, ABI>(g, mode, dag, pout, colour, out, in, U, a, x, c, nsites, abi);
 }
 
 // the double-float sweep: its long dependent chains want more resident
@@ -162,47 +236,52 @@ __global__ void __launch_bounds__(HOP_BS_MAX) k_hop(Geo g, int mode, int dag, in
 __global__ void __launch_bounds__(HOP_BS_MAX, 2) k_hop_df(Geo g, int mode, int dag, int pout, int colour, SpinorF out,
                                                      SpinorF in, GaugeF U, double a, SpinorF x, double c, int nsites)
 {
-    hop_body<PRECDF>(g, mode, dag, pout, colour, out, in, U, a, x, c, nsites);
+    hop_body<PRECDF, false>(g, mode, dag, pout, colour, out, in, U, a, x, c, nsites, nullptr);
 }
 
 }  // namespace
 
 // algorithmic DRAM bytes of one output site: the output, the input site and
 // the eight links, each moved once (neighbour spinors reused from cache)
-double hop_site_bytes(int prec, bool with_x)
+double hop_site_bytes(int prec, bool with_x, bool abi)
 {
     const bool dbl = prec == PREC64 || prec == PRECDF;
     const double sp = dbl ? 192.0 : prec == PREC32 ? 96.0 : prec == PREC16 ? 52.0 : 48.0;
     const double lk = dbl ? 144.0 : prec == PREC32 ? 48.0 : 24.0;
-    return 2.0 * sp + 8.0 * lk + (with_x ? sp : 0.0);
+    return sp + (abi ? 192.0 : sp) + 8.0 * lk + (with_x ? sp : 0.0);
 }
 
 int hop_sweep(lqcd_ctx* h, int prec, int mode, int dag, int pout, int colour, SpinorF out, SpinorF in,
-              double a, SpinorF x, double c)
+              double a, SpinorF x, double c, double2* abi)
 {
     const Geo& g = h->g;
-    const int nsites = colour < 0 ? g.Vh : (g.nb / 2) * g.Sh;
-    const int bs = std::min(std::max(h->tune.hop_bs[prec == PRECDF ? PREC64 : prec], 32), HOP_BS_MAX);
+    const int nsites = colour < 0 || abi ? g.Vh : (g.nb / 2) * g.Sh;
+    const int bs = std::min(std::max(h->tune.hop_bs[prec == PRECDF ? PREC64 : prec], 32), HOP_BS_MAX);  // whole warps
     const int nb = (nsites + bs - 1) / bs;
     GaugeF U = gauge_view(h, prec);
     cudaEvent_t ev;
     prof_begin(h, 0, &ev);
-    if (prec == PREC64)
-        k_hop<PREC64><<<nb, bs, 0, h->stream>>>(g, mode, dag, pout, colour, out, in, U, a, x, c, nsites);
+#define HOP(P)                                                                                                     \
+    do {                                                                                                           \
+        if (abi)                                                                                                   \
+            k_hop<P, true><<<nb, bs, abi_smem<P>(bs), h->stream>>>(g, mode, dag, pout, colour, out, in, U, a, x, c, \
+                                                                   nsites, abi);                                   \
+        else                                                                                                       \
+            k_hop<P, false><<<nb, bs, 0, h->stream>>>(g, mode, dag, pout, colour, out, in, U, a, x, c, nsites, abi); \
+    } while (0)
+    if (prec == PREC64) HOP(PREC64);
     else if (prec == PRECDF)
         k_hop_df<<<nb, bs, 0, h->stream>>>(g, mode, dag, pout, colour, out, in, U, a, x, c, nsites);
-    else if (prec == PREC32)
-        k_hop<PREC32><<<nb, bs, 0, h->stream>>>(g, mode, dag, pout, colour, out, in, U, a, x, c, nsites);
-    else if (prec == PREC16)
-        k_hop<PREC16><<<nb, bs, 0, h->stream>>>(g, mode, dag, pout, colour, out, in, U, a, x, c, nsites);
-    else
-        k_hop<PRECBF><<<nb, bs, 0, h->stream>>>(g, mode, dag, pout, colour, out, in, U, a, x, c, nsites);
+    else if (prec == PREC32) HOP(PREC32);
+    else if (prec == PREC16) HOP(PREC16);
+    else HOP(PRECBF);
+#undef HOP
     h->launches += 1;
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
         h->err = std::string("hop kernel: ") + cudaGetErrorString(e);
         return LQCD_ERR_CUDA;
     }
-    prof_end(h, 0, ev, hop_site_bytes(prec, x.v != nullptr) * nsites);
+    prof_end(h, 0, ev, hop_site_bytes(prec, x.v != nullptr, abi != nullptr) * nsites);
     return LQCD_OK;
 }

@@ -24,6 +24,38 @@ __global__ void k_pack_spinor(double2* dst, const double2* abi, int Vh, int par0
     for (int c = 0; c < 12; ++c) d[(size_t)c * Vh + i] = a[c];
 }
 
+// C-ABI spinors straight into the storage of a single- or half-precision
+// sweep.  A warp reads its 32 sites along the field (6 KB in a row) and hands
+// each lane its site through shared memory, rounded to float on the way (as
+// a separate conversion of the packed doubles did).
+template <int P>
+__global__ void __launch_bounds__(128) k_pack_low(SpinorF dst, const double2* abi, int Vh)
+{
+    __shared__ float2 sh[4][32 * 13];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int s0 = (blockIdx.x * 4 + w) * 32;
+    const int n = min(32, Vh - s0);
+    if (n <= 0) return;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+        const int e = k * 32 + lane;
+        if (e < 12 * n) {
+            const double2 v = __ldg(abi + (size_t)s0 * 12 + e);
+            sh[w][e / 12 * 13 + e % 12] = make_float2((float)v.x, (float)v.y);
+        }
+    }
+    __syncwarp();
+    if (lane < n) {
+        Spinor<float> s;
+#pragma unroll
+        for (int c = 0; c < 12; ++c) {
+            const float2 v = sh[w][lane * 13 + c];
+            s.c[c / 3][c % 3] = mk(v.x, v.y);
+        }
+        store_spinor<P>(dst, s0 + lane, s);
+    }
+}
+
 __global__ void k_unpack_spinor(double2* abi, const double2* src, int Vh, int par0, int npar)
 {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -392,6 +424,20 @@ int unpack_spinor(lqcd_ctx* h, double* abi, const double2* src, int par0, int np
     k_unpack_spinor<<<nblk((int64_t)npar * Vh), BS, 0, h->stream>>>((double2*)abi, src, Vh, par0, npar);
     LAUNCH_CHECK(h);
     prof_end(h, 4, ev, 2.0 * 192.0 * npar * Vh);
+    return LQCD_OK;
+}
+
+int pack_spinor_low(lqcd_ctx* h, SpinorF dst, int prec, const double* abi)
+{
+    const int Vh = h->g.Vh, nb = nblk(Vh, 128);
+    const double2* a = (const double2*)abi;
+    cudaEvent_t ev;
+    prof_begin(h, 4, &ev);
+    if (prec == PREC32) k_pack_low<PREC32><<<nb, 128, 0, h->stream>>>(dst, a, Vh);
+    else if (prec == PREC16) k_pack_low<PREC16><<<nb, 128, 0, h->stream>>>(dst, a, Vh);
+    else k_pack_low<PRECBF><<<nb, 128, 0, h->stream>>>(dst, a, Vh);
+    LAUNCH_CHECK(h);
+    prof_end(h, 4, ev, (192.0 + (prec == PREC32 ? 96.0 : prec == PREC16 ? 52.0 : 48.0)) * Vh);
     return LQCD_OK;
 }
 

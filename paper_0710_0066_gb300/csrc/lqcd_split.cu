@@ -369,11 +369,10 @@ __device__ __forceinline__ cx<double> link_entry(const double2 (&l)[9], int r, i
 }
 __device__ __forceinline__ cx<double> link_row2(const double2 (&l)[9], int c) { return link_entry(l, 2, c); }
 
-// a b + c, with one rounding per product
-template <class T>
-__device__ __forceinline__ cx<T> cfma(cx<T> a, cx<T> b, cx<T> c)
+using ::cfma;
+__device__ __forceinline__ cx<float> cfma(cx<float> a, cx<float> b, cx<float> c)
 {
-    return mk(fma(-a.im, b.im, fma(a.re, b.re, c.re)), fma(a.im, b.re, fma(a.re, b.im, c.im)));
+    return mk(fmaf(-a.im, b.im, fmaf(a.re, b.re, c.re)), fmaf(a.im, b.re, fmaf(a.re, b.im, c.im)));
 }
 template <class T>
 __device__ __forceinline__ cx<T> cmul1(cx<T> a, cx<T> b)

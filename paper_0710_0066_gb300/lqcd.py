@@ -422,6 +422,13 @@ class Lattice:
         except Exception:
             pass
 
+    # results that a call writes in full need no clearing pass
+    def _spinor_out(self):
+        return torch.empty((self.V, 4, 3), dtype=torch.complex128, device=self.dev)
+
+    def _half_out(self):
+        return torch.empty((self.Vh, 4, 3), dtype=torch.complex128, device=self.dev)
+
     def spinor(self):
         return torch.zeros((self.V, 4, 3), dtype=torch.complex128, device=self.dev)
 
@@ -451,40 +458,40 @@ class Lattice:
         return m
 
     def dslash_eo(self, x, parity, kappa=0.0, dagger=0, op=OP_HOP, precision=PREC_F64):
-        out = self.half()
+        out = self._half_out()
         lqcd_dslash_eo(self.h, out, x.contiguous(), kappa, parity, dagger, op, precision)
         return out
 
     def block_dslash(self, x, kappa, colour=-1, dagger=0, precision=PREC_F64):
-        out = self.spinor()
+        out = self._spinor_out()
         lqcd_block_dslash(self.h, out, x.contiguous(), kappa, colour, dagger, precision)
         return out
 
     def block_solve(self, b, kappa, colour=-1, dagger=0, precision=PREC_F64, tol=1e-10, max_iter=10000):
-        x = self.spinor()
+        x = self._spinor_out()
         it, rs = lqcd_block_solve_batched(self.h, x, b.contiguous(), kappa, colour, dagger, precision,
                                           tol, max_iter, nb=self.nb)
         return x, it, rs
 
     def subblock_dslash(self, x, kappa, colour=-1, dagger=0, precision=PREC_F64):
-        out = self.spinor()
+        out = self._spinor_out()
         lqcd_subblock_dslash(self.h, out, x.contiguous(), kappa, colour, dagger, precision)
         return out
 
     def subblock_solve(self, b, kappa, colour=-1, dagger=0, precision=PREC_F64, tol=1e-10, max_iter=10000):
-        x = self.spinor()
+        x = self._spinor_out()
         it, rs = lqcd_subblock_solve_batched(self.h, x, b.contiguous(), kappa, colour, dagger, precision,
                                              tol, max_iter, nbs=self.nbs)
         return x, it, rs
 
     def w3eo(self, x_e, kappa, rho, dagger=0):
-        out = self.half()
+        out = self._half_out()
         lqcd_subblock_eo(self.h, out, x_e.contiguous(), kappa, rho, dagger, EO_APPLY, nbs=self.nbs)
         return out
 
     def solve_w3eo(self, b_e, kappa, rho, dagger=0, precision=PREC_F64, tol=1e-10, max_iter=10000,
                    method=SOLVER_BICGSTAB):
-        x = self.half()
+        x = self._half_out()
         it = lqcd_subblock_eo(self.h, x, b_e.contiguous(), kappa, rho, dagger, EO_SOLVE, precision, tol, max_iter,
                               nbs=self.nbs, method=method)
         return x, it
@@ -495,7 +502,7 @@ class Lattice:
         return S, F
 
     def solve(self, b, kappa, dagger=0, precision=PREC_F64, tol=1e-10, max_iter=20000):
-        x = self.spinor()
+        x = self._spinor_out()
         it, rs = lqcd_solve_wilson(self.h, x, b.contiguous(), kappa, dagger, precision, tol, max_iter)
         return x, it, rs
 
