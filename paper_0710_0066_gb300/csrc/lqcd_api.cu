@@ -1295,8 +1295,12 @@ int lqcd_gauge_force(lqcd_t h, double* F, double beta, double* S_out, double* pl
 {
     CHECK_H(h);
     NEED_GAUGE(h);
-    if (F) LQ_TRY(gauge_force_kick(h, F, beta / 6.0, PREC64));
-    LQ_TRY(plaquette_sum(h, h->red_out));
+    if (F) {
+        double2* const scratch[3] = {fld(h, F_A), fld(h, F_B), fld(h, F_C)};
+        LQ_TRY(gauge_force_action(h, F, beta / 6.0, scratch, h->red_out));
+    } else {
+        LQ_TRY(plaquette_sum(h, h->red_out));
+    }
     double s;
     LQ_TRY(read_scalars(h, 1, &s));
     if (S_out) *S_out = -beta / 3.0 * s;

@@ -1185,6 +1185,9 @@ int force_bilinear(lqcd_ctx* h, double* F, const double2* a1, const double2* b1,
                    double coef1, const double2* a2, const double2* b2, int mask2, double coef2, int prec,
                    const double* ss = nullptr);
 int gauge_force_kick(lqcd_ctx* h, double* F, double coef, int prec, const double* ss = nullptr);
+// F += coef 2 Im tr(T^a U A) of every link in double precision and the
+// plaquette sum in one go; scratch: three full double fields
+int gauge_force_action(lqcd_ctx* h, double* F, double coef, double2* const* scratch, double* dev_out);
 int plaquette_sum(lqcd_ctx* h, double* dev_out);
 int force_profile(lqcd_ctx* h, const double* F, double* out);
 int update_links(lqcd_ctx* h, const double* P, double dt, const double* ss = nullptr);

@@ -53,7 +53,7 @@ __device__ __forceinline__ void su3_mul(const Su3<T>& a, const Su3<T>& b, Su3<T>
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
-        for (int j = 0; j < 3; ++j) c.m[i][j] = a.m[i][0] * b.m[0][j] + a.m[i][1] * b.m[1][j] + a.m[i][2] * b.m[2][j];
+        for (int j = 0; j < 3; ++j) c.m[i][j] = cdot3(a.m[i][0], b.m[0][j], a.m[i][1], b.m[1][j], a.m[i][2], b.m[2][j]);
 }
 // c = a b^dag
 template <class T>
@@ -63,7 +63,7 @@ __device__ __forceinline__ void su3_mul_nd(const Su3<T>& a, const Su3<T>& b, Su3
     for (int i = 0; i < 3; ++i)
 #pragma unroll
         for (int j = 0; j < 3; ++j)
-            c.m[i][j] = a.m[i][0] * conjx(b.m[j][0]) + a.m[i][1] * conjx(b.m[j][1]) + a.m[i][2] * conjx(b.m[j][2]);
+            c.m[i][j] = cdot3(a.m[i][0], conjx(b.m[j][0]), a.m[i][1], conjx(b.m[j][1]), a.m[i][2], conjx(b.m[j][2]));
 }
 
 template <class T>
@@ -246,6 +246,17 @@ __global__ void __launch_bounds__(BS) k_gauge_force(Geo g, GaugeF U, double* F, 
     for (int k = 0; k < 8; ++k) d[k] += c * l[k];
 }
 
+// Re tr a b^dag
+__device__ __forceinline__ double retr_nd(const Su3<double>& a, const Su3<double>& b)
+{
+    double v = 0.0;
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) v = fma(a.m[i][j].im, b.m[i][j].im, fma(a.m[i][j].re, b.m[i][j].re, v));
+    return v;
+}
+
 __device__ __forceinline__ double block_sum(double v)
 {
     __shared__ double sh[32];
@@ -284,14 +295,167 @@ __global__ void k_plaq_part(Geo g, GaugeF U, double* part)
                 site_at(g, y, p, j);
                 load_link<PREC64>(U, mu, p, j, c);
                 load_link<PREC64>(U, nu, par, i, d);
+                // Re tr (a b) (d c)^dag: two products and a trace
                 su3_mul(a, b, t);
-                su3_mul_nd(t, c, r);
-                su3_mul_nd(r, d, t);
-                acc += t.m[0][0].re + t.m[1][1].re + t.m[2][2].re;
+                su3_mul(d, c, r);
+                acc += retr_nd(t, r);
             }
     }
     acc = block_sum(acc);
     if (threadIdx.x == 0) part[blockIdx.x] = acc;
+}
+
+// ---------------------------------------------------------------------------
+// The double-precision gauge force with the action (lqcd_gauge_force).  Bound
+// by FP64 instructions (two lanes per cycle and SM), so every plaquette is
+// multiplied out once: k_plaq_h forms P = U_mu(x) U_nu(x+mu) (U_nu(x) U_mu(x+nu))^dag
+// per plane (three products, 324 instructions), its trace for the action, and
+// keeps i (P^dag - P), hermitian, as nine numbers.  A link's force is the sum
+// over its planes of that matrix at x (the sign turned for the second
+// direction) and of the one at x - nu carried to x by U_nu(x - nu)^dag . U_nu(x - nu),
+// 162 instructions for a hermitian matrix.  3900 FP64 instructions a site
+// against 7400 of the staple form and its separate plaquette sum.
+// 32x16^3: 2.45 -> 1.02 ms a call (the staple form and the plaquette sum, both
+// before the fused multiply-adds of cdot3, against this).
+// ---------------------------------------------------------------------------
+constexpr int PLANE_W = 9;  // numbers per plane and site
+struct PlaneH {             // [plane][9][V], two planes per buffer
+    double* b[3];
+    __device__ __forceinline__ double* at(int V, int pl) const { return b[pl >> 1] + (size_t)(pl & 1) * PLANE_W * V; }
+};
+
+__device__ __forceinline__ int plane_of(int mu, int nu)  // mu > nu
+{
+    return mu * (mu - 1) / 2 + nu;
+}
+
+// of a plane's nine numbers: the diagonal, then (re, im) of entries 01, 02, 12
+__global__ void __launch_bounds__(BS) k_plaq_h(Geo g, GaugeF U, PlaneH H, double* part)
+{
+    double acc = 0.0;
+    // one item per plane and site; the sums in a fixed order
+    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < (int64_t)6 * g.V;
+         t += (int64_t)gridDim.x * blockDim.x) {
+        const int pl = (int)(t / g.V), s = (int)(t - (int64_t)pl * g.V);
+        const int mu = pl == 0 ? 1 : pl < 3 ? 2 : 3, nu = pl - mu * (mu - 1) / 2;
+        const int par = s >= g.Vh ? 1 : 0, i = s - par * g.Vh;
+        int x[4], y[4], p, j;
+        eo_coords(g, par, i, x);
+        Su3<double> a, b, t1, t2;
+        load_link<PREC64>(U, mu, par, i, a);
+        shifted(g, x, mu, +1, y);
+        site_at(g, y, p, j);
+        load_link<PREC64>(U, nu, p, j, b);
+        su3_mul(a, b, t1);
+        load_link<PREC64>(U, nu, par, i, a);
+        shifted(g, x, nu, +1, y);
+        site_at(g, y, p, j);
+        load_link<PREC64>(U, mu, p, j, b);
+        su3_mul(a, b, t2);
+        su3_mul_nd(t1, t2, a);  // P
+        acc += a.m[0][0].re + a.m[1][1].re + a.m[2][2].re;
+        double* h = H.at(g.V, pl) + s;
+        // i (P^dag - P): diagonal 2 Im P_kk, entry jk of the upper triangle
+        // i (conj(P_kj) - P_jk)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) h[(size_t)k * g.V] = 2.0 * a.m[k][k].im;
+        int e = 3;
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+#pragma unroll
+            for (int c = r + 1; c < 3; ++c) {
+                h[(size_t)e++ * g.V] = a.m[c][r].im + a.m[r][c].im;
+                h[(size_t)e++ * g.V] = a.m[c][r].re - a.m[r][c].re;
+            }
+    }
+    acc = block_sum(acc);
+    if (threadIdx.x == 0) part[blockIdx.x] = acc;
+}
+
+struct Herm {
+    double d[3];
+    cx<double> o[3];  // entries 01, 02, 12
+};
+
+__device__ __forceinline__ void load_herm(const PlaneH& H, int V, int pl, int s, Herm& h)
+{
+    const double* p = H.at(V, pl) + s;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) h.d[k] = __ldg(p + (size_t)k * V);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) h.o[k] = mk(__ldg(p + (size_t)(3 + 2 * k) * V), __ldg(p + (size_t)(4 + 2 * k) * V));
+}
+
+// f += u^dag h u
+__device__ __forceinline__ void carry(const Su3<double>& u, const Herm& h, double sg, Herm& f)
+{
+    Su3<double> t;  // h u
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const cx<double> u0 = u.m[0][c], u1 = u.m[1][c], u2 = u.m[2][c];
+        t.m[0][c] = cfma(h.o[1], u2, cfma(h.o[0], u1, h.d[0] * u0));
+        t.m[1][c] = cfma(h.o[2], u2, cjfma(h.o[0], u0, h.d[1] * u1));
+        t.m[2][c] = cjfma(h.o[2], u1, cjfma(h.o[1], u0, h.d[2] * u2));
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        double v = 0.0;
+#pragma unroll
+        for (int r = 0; r < 3; ++r) v = fma(u.m[r][k].im, t.m[r][k].im, fma(u.m[r][k].re, t.m[r][k].re, v));
+        f.d[k] = fma(sg, v, f.d[k]);
+    }
+    int e = 0;
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int c = a + 1; c < 3; ++c, ++e) {
+            const cx<double> v = cjdot3(u.m[0][a], t.m[0][c], u.m[1][a], t.m[1][c], u.m[2][a], t.m[2][c]);
+            f.o[e] = mk(fma(sg, v.re, f.o[e].re), fma(sg, v.im, f.o[e].im));
+        }
+}
+
+// F += c 2 Im tr(T^a Y), Y the sum of the link's six plaquettes: with the
+// hermitian h = i (Y^dag - Y) that is c times (h_01 re, -h_01 im, ..) below
+__global__ void __launch_bounds__(BS) k_gauge_force_h(Geo g, GaugeF U, PlaneH H, double* F, double c)
+{
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= 4 * g.V) return;
+    const int mu = t / g.V, s = t - mu * g.V;
+    const int par = s >= g.Vh ? 1 : 0, i = s - par * g.Vh;
+    int x[4];
+    eo_coords(g, par, i, x);
+    Herm f;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        f.d[k] = 0.0;
+        f.o[k] = mk(0.0, 0.0);
+    }
+#pragma unroll 1
+    for (int nu = 0; nu < 4; ++nu) {
+        if (nu == mu) continue;
+        const int pl = mu > nu ? plane_of(mu, nu) : plane_of(nu, mu);
+        const double sg = mu > nu ? 1.0 : -1.0;
+        Herm h;
+        load_herm(H, g.V, pl, s, h);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            f.d[k] = fma(sg, h.d[k], f.d[k]);
+            f.o[k] = mk(fma(sg, h.o[k].re, f.o[k].re), fma(sg, h.o[k].im, f.o[k].im));
+        }
+        int y[4], p, j;
+        shifted(g, x, nu, -1, y);
+        site_at(g, y, p, j);
+        Su3<double> u;
+        load_link<PREC64>(U, nu, p, j, u);
+        load_herm(H, g.V, pl, p * g.Vh + j, h);
+        // the plaquette below the link runs against it: the opposite sign
+        carry(u, h, -sg, f);
+    }
+    double* d = F + ((size_t)mu * g.V + s) * 8;
+    const double l[8] = {f.o[0].re, -f.o[0].im, 0.5 * (f.d[0] - f.d[1]), f.o[1].re, -f.o[1].im,
+                         f.o[2].re, -f.o[2].im, 0.5 * (f.d[0] + f.d[1] - 2.0 * f.d[2]) * INV_SQRT3};
+#pragma unroll
+    for (int k = 0; k < 8; ++k) d[k] += c * l[k];
 }
 
 __global__ void k_sum_final(const double* part, int n, double* out, double scale)
@@ -625,6 +789,23 @@ int gauge_force_kick(lqcd_ctx* h, double* F, double coef, int prec, const double
         k_gauge_force<PREC32><<<nb, BS, 0, h->stream>>>(h->g, gauge_view(h, PREC32), F, coef, ss);
     LQ_TRY(launch_err(h, "gauge force kernel"));
     prof_end(h, 3, ev, (double)h->g.V * (4.0 * 144.0 + 2.0 * 256.0));
+    return LQCD_OK;
+}
+
+int gauge_force_action(lqcd_ctx* h, double* F, double coef, double2* const* scratch, double* dev_out)
+{
+    PlaneH H;
+    for (int k = 0; k < 3; ++k) H.b[k] = (double*)scratch[k];
+    cudaEvent_t ev;
+    prof_begin(h, 3, &ev);
+    const int nb = (4 * h->g.V + BS - 1) / BS;
+    k_plaq_h<<<h->red_blocks, BS, 0, h->stream>>>(h->g, gauge_view(h, PREC64), H, h->red_part);
+    LQ_TRY(launch_err(h, "plaquette kernel"));
+    k_sum_final<<<1, 1024, 0, h->stream>>>(h->red_part, h->red_blocks, dev_out, 1.0);
+    LQ_TRY(launch_err(h, "plaquette sum"));
+    k_gauge_force_h<<<nb, BS, 0, h->stream>>>(h->g, gauge_view(h, PREC64), H, F, coef);
+    LQ_TRY(launch_err(h, "gauge force kernel"));
+    prof_end(h, 3, ev, (double)h->g.V * (2.0 * 4.0 * 144.0 + 3.0 * 6.0 * 72.0 + 2.0 * 256.0));
     return LQCD_OK;
 }
 
