@@ -13,8 +13,8 @@
 // Doubles are split into df with integer operations only (no conversion
 // through the FP64 pipe): hi takes the sign, the exponent and the leading
 // 23 fraction bits; lo the next 23 of the remaining 29 fraction bits, so
-// the split is exact to a relative 2^-46.  Values below 2^-126 in
-// magnitude (and zeros) split to hi only; below 2^-80 lo is dropped.
+// the split is exact to a relative 2^-46.  Values below 2^-80 in magnitude
+// (and zeros) split to hi only.
 // Results go back to double as (double) hi + (double) lo.
 //
 // Every function is host- and device-callable so that the host compiler
@@ -123,23 +123,37 @@ LQ_HD df df_norm(df a)
     return r;
 }
 
+// Nine instructions for the pair and four for the range: a df sweep splits
+// 336 doubles a site.
 LQ_HD df df_split(double x)
 {
     const uint64_t b = df_bits64(x);
-    const uint32_t sign = (uint32_t)(b >> 32) & 0x80000000u;
-    const int e = (int)((b >> 52) & 0x7ff);  // biased double exponent
-    if (e == 0) return df(0.f, 0.f);        // zero (and double subnormals)
-    const int ef = e - 1023 + 127;           // biased float exponent of hi
-    if (ef <= 0 || ef >= 255) return df((float)x, 0.f);  // outside the float range, inf, nan
-    const float h = df_f32(sign | ((uint32_t)ef << 23) | (uint32_t)((b >> 29) & 0x7fffffu));
+    const uint32_t top = (uint32_t)(b >> 32), low = (uint32_t)b;
+    // the leading 32 bits below sign and two exponent bits, the exponent e
+    // taken from the double's bias to the float's: for 897 <= e <= 1150
+    const uint32_t hb = (((uint32_t)(b >> 29) + 0x40000000u) & 0x7fffffffu) | (top & 0x80000000u);
     // remainder: the low 29 fraction bits m, worth m 2^(e - 1075); keep the
     // top 23 (m23 = m >> 6, worth m23 2^(e - 1069)).  float(m23) is exact:
-    // 2^23 + m23 has the float bit pattern 0x4B000000 | m23.
-    const uint32_t m23 = (uint32_t)(b & 0x1fffffffu) >> 6;
-    float l = df_f32(0x4B000000u | m23) - 8388608.0f;
-    const int es = e - 1069 + 127;  // biased float exponent of 2^(e - 1069)
-    l = es > 0 ? l * df_f32((uint32_t)es << 23) : 0.f;
-    return df(h, sign ? -l : l);
+    // 2^23 + m23 has the float bit pattern 0x4B000000 | m23.  The factor
+    // 2^(e - 1069), with the sign, is hi's exponent less 46.
+    float h = df_f32(hb);
+    float l = (df_f32(((low >> 6) & 0x7fffffu) | 0x4B000000u) - 8388608.0f) *
+              df_f32((hb & 0xff800000u) - (46u << 23));
+    // outside 2^-80 <= |x| < 2^128 (zero, tiny, inf, nan): the nearest float
+    const uint32_t range = (top & 0x7fffffffu) - (943u << 20);
+#ifdef __CUDA_ARCH__
+    // (predicated: a branch per number would break the loads and the
+    // arithmetic around it into pieces)
+    asm("{\n\t.reg .pred p;\n\tsetp.ge.u32 p, %2, %3;\n\t@p cvt.rn.f32.f64 %0, %4;\n\t@p mov.f32 %1, 0f00000000;\n\t}"
+        : "+f"(h), "+f"(l)
+        : "r"(range), "r"(208u << 20), "d"(x));
+#else
+    if (range >= (208u << 20)) {
+        h = (float)x;
+        l = 0.f;
+    }
+#endif
+    return df(h, l);
 }
 
 LQ_HD double df_to_double(df a) { return (double)a.hi + (double)a.lo; }
