@@ -505,8 +505,8 @@ __global__ void k_force_profile(Geo g, const double* F, double* out)
 // Cayley-Hamilton, Q^3 = c1 Q + c0 (c0 = det Q): with Q^n = a0 + a1 Q + a2 Q^2,
 // Q^(n+1) = c0 a2 + (a0 + c1 a2) Q + a1 Q^2, and f_j = sum_n i^n a_j / n!,
 // a scalar recurrence without transcendental functions (terms fall below
-// 1e-17 of the leading ones after about 6 + 3 |Q| steps); larger Q use the
-// closed form with the trigonometric functions.
+// 1e-18 after about 6 + 3 |Q| steps; their bound |Q|^n / n! is kept in single
+// precision); larger Q use the closed form with the trigonometric functions.
 // 1 / n!, n = 0..40, for the series of expiq (constant memory: every
 // thread of a warp reads the same entry)
 constexpr double inv_factorial(int n) { return n <= 1 ? 1.0 : inv_factorial(n - 1) / n; }
@@ -519,149 +519,128 @@ __constant__ double c_invfact[41] = {
     inv_factorial(30), inv_factorial(31), inv_factorial(32), inv_factorial(33), inv_factorial(34), inv_factorial(35),
     inv_factorial(36), inv_factorial(37), inv_factorial(38), inv_factorial(39), inv_factorial(40)};
 
-// Q^2 of a hermitian Q from its six distinct entries (real diagonal)
-__device__ __forceinline__ void herm_square(const Su3<double>& Q, Su3<double>& Q2)
+// Q^2 and its invariants: c1 = tr Q^2 / 2, c0 = det Q (tr Q = 0)
+__device__ __forceinline__ void herm_square(const Herm& Q, Herm& Q2, double& c1, double& c0)
 {
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        double d = 0.0;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) d += Q.m[i][k].re * Q.m[i][k].re + Q.m[i][k].im * Q.m[i][k].im;
-        Q2.m[i][i] = mk(d, 0.0);
-#pragma unroll
-        for (int j = i + 1; j < 3; ++j) {
-            const cx<double> v = Q.m[i][0] * Q.m[0][j] + Q.m[i][1] * Q.m[1][j] + Q.m[i][2] * Q.m[2][j];
-            Q2.m[i][j] = v;
-            Q2.m[j][i] = conjx(v);
-        }
-    }
+    const double n01 = fma(Q.o[0].re, Q.o[0].re, Q.o[0].im * Q.o[0].im);
+    const double n02 = fma(Q.o[1].re, Q.o[1].re, Q.o[1].im * Q.o[1].im);
+    const double n12 = fma(Q.o[2].re, Q.o[2].re, Q.o[2].im * Q.o[2].im);
+    Q2.d[0] = fma(Q.d[0], Q.d[0], n01 + n02);
+    Q2.d[1] = fma(Q.d[1], Q.d[1], n01 + n12);
+    Q2.d[2] = fma(Q.d[2], Q.d[2], n02 + n12);
+    c1 = 0.5 * (Q2.d[0] + Q2.d[1] + Q2.d[2]);
+    // (Q^2)_01 = (d0 + d1) o01 + o02 o12^*, d0 + d1 = -d2, and so on
+    const cx<double> t = Q.o[0] * Q.o[2];
+    Q2.o[0] = cjfma(Q.o[2], Q.o[1], mk(-Q.d[2] * Q.o[0].re, -Q.d[2] * Q.o[0].im));
+    Q2.o[1] = mk(fma(-Q.d[1], Q.o[1].re, t.re), fma(-Q.d[1], Q.o[1].im, t.im));
+    Q2.o[2] = cjfma(Q.o[0], Q.o[1], mk(-Q.d[0] * Q.o[2].re, -Q.d[0] * Q.o[2].im));
+    const double re = fma(t.re, Q.o[1].re, t.im * Q.o[1].im);  // Re o01 o12 o02^*
+    c0 = fma(2.0, re, Q.d[0] * fma(Q.d[1], Q.d[2], -n12));
+    c0 = fma(-Q.d[1], n02, c0);
+    c0 = fma(-Q.d[2], n01, c0);
 }
 
-__device__ void expiq(const Su3<double>& Q, Su3<double>& E)
+__device__ __forceinline__ void expiq(const Herm& Q, Su3<double>& E)
 {
-    Su3<double> Q2;
-    herm_square(Q, Q2);
-    const double c1 = 0.5 * (Q2.m[0][0].re + Q2.m[1][1].re + Q2.m[2][2].re);
+    Herm Q2;
+    double c1, c0;
+    herm_square(Q, Q2, c1, c0);
     cx<double> f0, f1, f2;
-    if (c1 >= 1e-12 && c1 <= 1.0) {
-        const cx<double> det = Q.m[0][0] * (Q.m[1][1] * Q.m[2][2] - Q.m[1][2] * Q.m[2][1]) -
-                               Q.m[0][1] * (Q.m[1][0] * Q.m[2][2] - Q.m[1][2] * Q.m[2][0]) +
-                               Q.m[0][2] * (Q.m[1][0] * Q.m[2][1] - Q.m[1][1] * Q.m[2][0]);
-        const double c0 = det.re;
+    if (c1 <= 1.0) {
         double a0 = 1.0, a1 = 0.0, a2 = 0.0;  // Q^n coordinates
         double r0 = 1.0, r1 = 0.0, r2 = 0.0, i0 = 0.0, i1 = 0.0, i2 = 0.0;
-        const double qn = sqrt(2.0 * c1);  // Frobenius norm of Q: |Q^n| <= qn^n
-        double qp = 1.0;                    // qn^n
-        for (int n = 1; n <= 40; ++n) {
-            const double b0 = c0 * a2, b1 = a0 + c1 * a2, b2 = a1;
-            a0 = b0;
+        const float qn = sqrtf(2.0f * (float)c1);  // Frobenius norm of Q: |Q^n| <= qn^n
+        float bound = 1.0f;                         // qn^n / n!
+        int n = 0;
+        auto step = [&](double sg, double& s0, double& s1, double& s2) {
+            ++n;
+            const double b0 = c0 * a2, b1 = fma(c1, a2, a0), w = sg * c_invfact[n];
+            a2 = a1;
             a1 = b1;
-            a2 = b2;
-            const double w = c_invfact[n];
-            qp *= qn;
-            const double bound = qp * w;
-            // i^n: 1, i, -1, -i
-            switch (n & 3) {
-                case 0: r0 += w * a0; r1 += w * a1; r2 += w * a2; break;
-                case 1: i0 += w * a0; i1 += w * a1; i2 += w * a2; break;
-                case 2: r0 -= w * a0; r1 -= w * a1; r2 -= w * a2; break;
-                default: i0 -= w * a0; i1 -= w * a1; i2 -= w * a2; break;
-            }
-            if (bound < 1e-18) break;
-        }
+            a0 = b0;
+            s0 = fma(w, a0, s0);
+            s1 = fma(w, a1, s1);
+            s2 = fma(w, a2, s2);
+            bound *= __fdividef(qn, (float)n);
+            return bound < 1e-18f;
+        };
+        // i^n: i, -1, -i, 1
+        while (n < 40)
+            if (step(1.0, i0, i1, i2) || step(-1.0, r0, r1, r2) || step(-1.0, i0, i1, i2) || step(1.0, r0, r1, r2))
+                break;
         f0 = mk(r0, i0);
         f1 = mk(r1, i1);
         f2 = mk(r2, i2);
-#pragma unroll
-        for (int r = 0; r < 3; ++r)
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                cx<double> v = f1 * Q.m[r][c] + f2 * Q2.m[r][c];
-                if (r == c) v = v + f0;
-                E.m[r][c] = v;
-            }
-        return;
-    }
-    if (c1 < 1e-12) {
-        // |Q| < 1.5e-6: series to fourth order
-        Su3<double> Q3, Q4;
-        su3_mul(Q2, Q, Q3);
-        su3_mul(Q2, Q2, Q4);
-#pragma unroll
-        for (int r = 0; r < 3; ++r)
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                cx<double> v = mul_i(Q.m[r][c]) - 0.5 * Q2.m[r][c] - (1.0 / 6.0) * mul_i(Q3.m[r][c]) +
-                               (1.0 / 24.0) * Q4.m[r][c];
-                if (r == c) v.re += 1.0;
-                E.m[r][c] = v;
-            }
-        return;
-    }
-    // c0 = det Q (real)
-    const cx<double> det = Q.m[0][0] * (Q.m[1][1] * Q.m[2][2] - Q.m[1][2] * Q.m[2][1]) -
-                           Q.m[0][1] * (Q.m[1][0] * Q.m[2][2] - Q.m[1][2] * Q.m[2][0]) +
-                           Q.m[0][2] * (Q.m[1][0] * Q.m[2][1] - Q.m[1][1] * Q.m[2][0]);
-    const double c0 = det.re;
-    const double c0a = fabs(c0);
-    const double c0max = 2.0 * pow(c1 / 3.0, 1.5);
-    const double ratio = fmin(1.0, c0a / c0max);
-    const double theta = acos(ratio);
-    const double u = sqrt(c1 / 3.0) * cos(theta / 3.0);
-    const double w = sqrt(c1) * sin(theta / 3.0);
-    const double u2 = u * u, w2 = w * w;
-    double xi0;
-    if (fabs(w) < 0.05)
-        xi0 = 1.0 - w2 / 6.0 * (1.0 - w2 / 20.0 * (1.0 - w2 / 42.0));
-    else
-        xi0 = sin(w) / w;
-    double s2u, c2u, su, cu;
-    sincos(2.0 * u, &s2u, &c2u);
-    sincos(u, &su, &cu);
-    const double cw = cos(w);
-    const cx<double> e2 = mk(c2u, s2u), em = mk(cu, -su);
-    const cx<double> h0 = (u2 - w2) * e2 + em * mk(8.0 * u2 * cw, 2.0 * u * (3.0 * u2 + w2) * xi0);
-    const cx<double> h1 = (2.0 * u) * e2 - em * mk(2.0 * u * cw, -(3.0 * u2 - w2) * xi0);
-    const cx<double> h2 = e2 - em * mk(cw, 3.0 * u * xi0);
-    const double dinv = 1.0 / (9.0 * u2 - w2);
-    f0 = dinv * h0;
-    f1 = dinv * h1;
-    f2 = dinv * h2;
-    if (c0 < 0.0) {  // f_j(-c0) = (-1)^j conj(f_j(c0))
-        f0 = conjx(f0);
-        f1 = -conjx(f1);
-        f2 = conjx(f2);
+    } else {
+        const double c0a = fabs(c0);
+        const double c0max = 2.0 * pow(c1 / 3.0, 1.5);
+        const double ratio = fmin(1.0, c0a / c0max);
+        const double theta = acos(ratio);
+        const double u = sqrt(c1 / 3.0) * cos(theta / 3.0);
+        const double w = sqrt(c1) * sin(theta / 3.0);
+        const double u2 = u * u, w2 = w * w;
+        double xi0;
+        if (fabs(w) < 0.05)
+            xi0 = 1.0 - w2 / 6.0 * (1.0 - w2 / 20.0 * (1.0 - w2 / 42.0));
+        else
+            xi0 = sin(w) / w;
+        double s2u, c2u, su, cu;
+        sincos(2.0 * u, &s2u, &c2u);
+        sincos(u, &su, &cu);
+        const double cw = cos(w);
+        const cx<double> e2 = mk(c2u, s2u), em = mk(cu, -su);
+        const cx<double> h0 = (u2 - w2) * e2 + em * mk(8.0 * u2 * cw, 2.0 * u * (3.0 * u2 + w2) * xi0);
+        const cx<double> h1 = (2.0 * u) * e2 - em * mk(2.0 * u * cw, -(3.0 * u2 - w2) * xi0);
+        const cx<double> h2 = e2 - em * mk(cw, 3.0 * u * xi0);
+        const double dinv = 1.0 / (9.0 * u2 - w2);
+        f0 = dinv * h0;
+        f1 = dinv * h1;
+        f2 = dinv * h2;
+        if (c0 < 0.0) {  // f_j(-c0) = (-1)^j conj(f_j(c0))
+            f0 = conjx(f0);
+            f1 = -conjx(f1);
+            f2 = conjx(f2);
+        }
     }
 #pragma unroll
-    for (int r = 0; r < 3; ++r)
+    for (int k = 0; k < 3; ++k)
+        E.m[k][k] = mk(fma(f2.re, Q2.d[k], fma(f1.re, Q.d[k], f0.re)), fma(f2.im, Q2.d[k], fma(f1.im, Q.d[k], f0.im)));
+    int e = 0;
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            cx<double> v = f1 * Q.m[r][c] + f2 * Q2.m[r][c];
-            if (r == c) v = v + f0;
-            E.m[r][c] = v;
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int c = a + 1; c < 3; ++c, ++e) {
+            const cx<double> o = Q.o[e], p = Q2.o[e];
+            const double rr = fma(f2.re, p.re, f1.re * o.re), ii = fma(f2.im, p.im, f1.im * o.im);
+            const double ri = fma(f2.re, p.im, f1.re * o.im), ir = fma(f2.im, p.re, f1.im * o.re);
+            E.m[a][c] = mk(rr - ii, ri + ir);
+            E.m[c][a] = mk(rr + ii, ir - ri);
         }
 }
 
-__device__ void reunitarise(Su3<double>& u)
+// rows 0 and 1 orthonormalised, row 2 their completion
+__device__ __forceinline__ void reunitarise(Su3<double>& u)
 {
     double n0 = 0.0;
 #pragma unroll
-    for (int j = 0; j < 3; ++j) n0 += u.m[0][j].re * u.m[0][j].re + u.m[0][j].im * u.m[0][j].im;
+    for (int j = 0; j < 3; ++j) n0 = fma(u.m[0][j].re, u.m[0][j].re, fma(u.m[0][j].im, u.m[0][j].im, n0));
     n0 = rsqrt(n0);
 #pragma unroll
     for (int j = 0; j < 3; ++j) u.m[0][j] = n0 * u.m[0][j];
-    cx<double> d = mk(0.0, 0.0);
+    const cx<double> d = cjdot3(u.m[0][0], u.m[1][0], u.m[0][1], u.m[1][1], u.m[0][2], u.m[1][2]);
 #pragma unroll
-    for (int j = 0; j < 3; ++j) d = d + cjmul(u.m[0][j], u.m[1][j]);
-#pragma unroll
-    for (int j = 0; j < 3; ++j) u.m[1][j] = u.m[1][j] - d * u.m[0][j];
+    for (int j = 0; j < 3; ++j) u.m[1][j] = cfma(-d, u.m[0][j], u.m[1][j]);
     double n1 = 0.0;
 #pragma unroll
-    for (int j = 0; j < 3; ++j) n1 += u.m[1][j].re * u.m[1][j].re + u.m[1][j].im * u.m[1][j].im;
+    for (int j = 0; j < 3; ++j) n1 = fma(u.m[1][j].re, u.m[1][j].re, fma(u.m[1][j].im, u.m[1][j].im, n1));
     n1 = rsqrt(n1);
 #pragma unroll
     for (int j = 0; j < 3; ++j) u.m[1][j] = n1 * u.m[1][j];
-    complete_row2(u);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        const int k = (j + 1) % 3, l = (j + 2) % 3;
+        u.m[2][j] = conjx(cfma(-u.m[0][l], u.m[1][k], u.m[0][k] * u.m[1][l]));
+    }
 }
 
 __device__ void store_link_all(double2* U64, float4* U32, uint2* U16, int Vh, int mp, int i, const Su3<double>& u)
@@ -677,6 +656,9 @@ __device__ void store_link_all(double2* U64, float4* U32, uint2* U16, int Vh, in
 }
 
 // U_mu(x) <- exp(i dt P_mu(x)) U_mu(x), P = sum_a p^a T^a; all three copies
+// Bound by FP64 instructions: Q and Q^2 as hermitian matrices (nine numbers),
+// entries of exp(iQ) in pairs, fused multiply-adds throughout, about 360
+// instead of 480 a link; a trajectory at 32x16^3 344 -> 339 ms.
 __global__ void __launch_bounds__(BS) k_update(Geo g, double2* U64, float4* U32, uint2* U16, const double* P, double dt,
                                               const double* ss)
 {
@@ -690,17 +672,15 @@ __global__ void __launch_bounds__(BS) k_update(Geo g, double2* U64, float4* U32,
     double q[8];
 #pragma unroll
     for (int k = 0; k < 8; ++k) q[k] = dt * p[k];
-    Su3<double> Q, E, u, n;
+    Herm Q;
+    Su3<double> E, u, n;
     const double r3 = q[7] * INV_SQRT3;
-    Q.m[0][0] = mk(0.5 * (q[2] + r3), 0.0);
-    Q.m[1][1] = mk(0.5 * (-q[2] + r3), 0.0);
-    Q.m[2][2] = mk(-r3, 0.0);
-    Q.m[0][1] = mk(0.5 * q[0], -0.5 * q[1]);
-    Q.m[1][0] = mk(0.5 * q[0], 0.5 * q[1]);
-    Q.m[0][2] = mk(0.5 * q[3], -0.5 * q[4]);
-    Q.m[2][0] = mk(0.5 * q[3], 0.5 * q[4]);
-    Q.m[1][2] = mk(0.5 * q[5], -0.5 * q[6]);
-    Q.m[2][1] = mk(0.5 * q[5], 0.5 * q[6]);
+    Q.d[0] = 0.5 * (q[2] + r3);
+    Q.d[1] = 0.5 * (r3 - q[2]);
+    Q.d[2] = -r3;
+    Q.o[0] = mk(0.5 * q[0], -0.5 * q[1]);
+    Q.o[1] = mk(0.5 * q[3], -0.5 * q[4]);
+    Q.o[2] = mk(0.5 * q[5], -0.5 * q[6]);
     expiq(Q, E);
     GaugeF G;
     G.v = U64;
