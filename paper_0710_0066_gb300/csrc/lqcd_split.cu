@@ -23,9 +23,9 @@
 //   * everywhere: FP64 issues two lanes per cycle and SM, so sums and scalars
 //     of a single-precision iteration are pairs of floats.
 // Measured (ms per solve to 1e-12, one thread per site without the above ->
-// this kernel): 12x6^3 global 4.48 -> 2.23, 32x16^3 global 33.8 -> 22.3, its
-// 8 slabs 4.85 -> 3.62, 64x32^3 global 695 -> 420, 32x24^3 series 9.28 -> 7.9;
-// double precision at 16x8^3 (two solves and the force) 34.8 -> 5.9.
+// this kernel): 12x6^3 global 5.06 -> 2.22, 32x16^3 global 30.2 -> 20.4, its
+// 8 slabs 4.80 -> 3.43, 64x32^3 global 647 -> 391, 32x24^3 series 9.23 -> 7.64;
+// double precision at 16x8^3 (two solves and the force) 34.5 -> 5.73.
 #include <algorithm>
 
 #include "lqcd_solve.cuh"
@@ -1167,6 +1167,23 @@ int pick(int prec, int groups, int num_sms)
     return groups <= 16 * num_sms ? V_1 : V_1W;
 }
 
+// How many of the systems a launch works on at a time.  Vectors and links that
+// an iteration of all of them reads and writes again may not fit the 129 MB L2
+// (96 bytes a vector and site, 384 the site's links); half as many at a time
+// do, and the sweeps are bound by L2 traffic.  Systems of 32x24^3 in slabs of
+// 8 (170 MB), series: four at a time 8.02 ms, two 7.64.  Not below the number
+// of groups at which one CTA per SM is filled: one at a time 10.3 ms.
+int systems_at_once(const SolveArgs& A, int prec, int method, int num_sms)
+{
+    constexpr double L2 = 129e6, FIT = 96e6;
+    const double set = (method == SOLVER_SERIES ? 4 * 96.0 + 384.0 : 6 * 96.0 + 384.0) * A.nsite;
+    if (prec != PREC32 || set * A.nsys <= L2) return A.nsys;
+    const int n = (int)(FIT / set);
+    if (n < 1) return A.nsys;
+    const int waves = (A.nsys + n - 1) / n, at = (A.nsys + waves - 1) / waves;
+    return (A.nsite + 31) / 32 * at >= 16 * num_sms ? at : A.nsys;
+}
+
 }  // namespace
 
 cudaError_t split_init(int num_sms, int occ[SPLIT_NVAR][2], int* gmax)
@@ -1187,11 +1204,11 @@ cudaError_t split_init(int num_sms, int occ[SPLIT_NVAR][2], int* gmax)
 SplitPlan split_plan(SolveArgs& A, int prec, int method, int spt, int num_sms, const int occ[SPLIT_NVAR][2])
 {
     const int G = (A.nsite + 31) / 32;
-    const int k = pick(prec, G * A.nsys, num_sms), m = method == SOLVER_SERIES ? 1 : 0;
+    A.ngrp = systems_at_once(A, prec, method, num_sms);
+    const int k = pick(prec, G * A.ngrp, num_sms), m = method == SOLVER_SERIES ? 1 : 0;
     const Variant& v = variants[k];
     const int SG = v.bs / 32 / v.lps;  // groups a CTA holds side by side
     const int want = spt <= 0 ? G : (G + SG * spt - 1) / (SG * spt);
-    A.ngrp = A.nsys;
     A.cps = std::max(1, std::min(occ[k][m] * num_sms / A.ngrp, want));
     const int gpc = (G + A.cps - 1) / A.cps;
     A.cps = (G + gpc - 1) / gpc;
