@@ -79,12 +79,12 @@ def thermalise_dynamical(lat, U, prm, ntraj, seed):
 PEAKS = os.path.join(ROOT, "MEASURED_PEAKS.json")
 
 # DRAM bytes per solver launch from the ncu capture summarised in
-# profiles/k_solve_16x16x16x32_f32.md, valid only for the solver source
+# profiles/k_split_16x16x16x32_f32.md, valid only for the solver source
 # that was captured (bench.py reports null once the source differs)
 SOLVER_SOURCES = ("lqcd_split.cu", "lqcd_solve.cuh", "lqcd_common.cuh", "lqcd_df.cuh")  # the sources k_split is built from
-SOLVER_TRAFFIC = dict(src_sha256="aef4788cc714dda78760d271604c272fd83e3842839fc76a07edbe1288dfd3b3",
-                      block_series=(303.767e6 + 154.127e6), block=(307.420e6 + 312.868e6),
-                      glob=(392.167e6 + 425.938e6))
+SOLVER_TRAFFIC = dict(src_sha256="d361f8bf57e40fdc75a5514e4db0ebe94ea8c46190e0eda92521a7be04447471",
+                      block_series=(346.314e6 + 147.963e6), block=(426.858e6 + 442.421e6),
+                      glob=(515.311e6 + 604.961e6))
 
 
 def solver_traffic():
@@ -103,7 +103,7 @@ def solver_traffic():
     return SOLVER_TRAFFIC["block_series"], {"batched_slab_solve_series": SOLVER_TRAFFIC["block_series"],
                                             "batched_slab_solve_bicgstab": SOLVER_TRAFFIC["block"],
                                             "global_solve_bicgstab": SOLVER_TRAFFIC["glob"],
-                                            "source": "profiles/k_solve_16x16x16x32_f32.md"}
+                                            "source": "profiles/k_split_16x16x16x32_f32.md"}
 
 
 def hbm_peak():
