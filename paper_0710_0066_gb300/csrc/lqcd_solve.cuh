@@ -5,7 +5,7 @@
 
 constexpr int NSYS_MAX = 64;
 constexpr int NQ = 3;
-constexpr int SPLIT_NQ = 8;  // partial sums per CTA in lqcd_split.cu
+constexpr int SPLIT_NQ = 4;  // partial sums per CTA in lqcd_split.cu
 constexpr int NACC = 5;  // iteration sums kept beside the sticky status
 
 // per-system state codes in the flag arrays

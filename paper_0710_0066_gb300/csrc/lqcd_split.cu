@@ -20,8 +20,10 @@
 //     sweep 1.5 times longer), vectors and links in tiles of 32 sites, no
 //     register spills (phases, barriers and reductions are kept apart for
 //     that: spilled registers tripled the L2 writes).
-//   * everywhere: FP64 issues two lanes per cycle and SM, so sums and scalars
-//     of a single-precision iteration are pairs of floats.
+//   * everywhere: the dot products of an iteration are FP64 sums and its
+//     scalars double, whatever the storage.  FP64 issues two lanes per cycle
+//     and SM, so a site's term (a word's, in an element-wise phase) is summed
+//     in the storage arithmetic first.
 // Measured (ms per solve to 1e-12, one thread per site without the above ->
 // this kernel): 12x6^3 global 5.06 -> 2.22, 32x16^3 global 30.2 -> 20.4, its
 // 8 slabs 4.80 -> 3.43, 64x32^3 global 647 -> 391, 32x24^3 series 9.23 -> 7.64;
@@ -33,14 +35,17 @@
 namespace {
 
 // ---------------------------------------------------------------------------
-// sums: single-precision terms accumulate in pairs of floats (the FP64 pipe
-// issues two lanes per cycle and SM: five shuffle steps of three FP64 sums
-// in every warp cost more than a hopping phase)
+// sums: FP64 over sites, warps and CTAs, of per-site terms in the storage
+// arithmetic.  The FP64 pipe issues two lanes per cycle and SM, so a sum
+// enters it as late as that allows.
 // ---------------------------------------------------------------------------
+// what a thread adds up in an element-wise phase, word by word: a pair of
+// floats in single precision (no FP64 instruction per word), one conversion
+// at the end
 template <class T>
-struct Acc;
+struct Local;
 template <>
-struct Acc<float> {
+struct Local<float> {
     float h, l;
     __device__ __forceinline__ void add(float x)
     {
@@ -49,45 +54,22 @@ struct Acc<float> {
         h = s;
         l += e;
     }
-    __device__ __forceinline__ void join(const Acc& o)
-    {
-        float s, e;
-        df_two_sum(h, o.h, s, e);
-        h = s;
-        l += o.l + e;
-    }
-    __device__ __forceinline__ Acc from(int m) const
-    {
-        return Acc{__shfl_xor_sync(0xffffffffu, h, m), __shfl_xor_sync(0xffffffffu, l, m)};
-    }
-    __device__ __forceinline__ Acc at(int k) const
-    {
-        return Acc{__shfl_sync(0xffffffffu, h, k), __shfl_sync(0xffffffffu, l, k)};
-    }
-    static __device__ __forceinline__ Acc zero() { return Acc{0.f, 0.f}; }
-    __device__ __forceinline__ double bits() const { return __hiloint2double(__float_as_int(l), __float_as_int(h)); }
-    static __device__ __forceinline__ Acc of(double d)
-    {
-        return Acc{__int_as_float(__double2loint(d)), __int_as_float(__double2hiint(d))};
-    }
+    __device__ __forceinline__ double value() const { return (double)h + (double)l; }
+    static __device__ __forceinline__ Local zero() { return Local{0.f, 0.f}; }
 };
 template <>
-struct Acc<double> {
+struct Local<double> {
     double h;
     __device__ __forceinline__ void add(double x) { h += x; }
-    __device__ __forceinline__ void join(const Acc& o) { h += o.h; }
-    __device__ __forceinline__ Acc from(int m) const { return Acc{__shfl_xor_sync(0xffffffffu, h, m)}; }
-    __device__ __forceinline__ Acc at(int k) const { return Acc{__shfl_sync(0xffffffffu, h, k)}; }
-    static __device__ __forceinline__ Acc zero() { return Acc{0.0}; }
-    __device__ __forceinline__ double bits() const { return h; }
-    static __device__ __forceinline__ Acc of(double d) { return Acc{d}; }
+    __device__ __forceinline__ double value() const { return h; }
+    static __device__ __forceinline__ Local zero() { return Local{0.0}; }
 };
 
-// warp sums of N = 1, 4 or 8 quantities, halving the quantities a lane
-// carries with every step (N = 8: nine joins instead of forty): every lane
-// returns the sum of quantity lane * N / 32
-template <int N, class A1>
-__device__ __forceinline__ A1 warp_sum(A1 (&v)[N])
+// warp sums of N = 1, 2 or 4 quantities, halving the quantities a lane
+// carries with every step (N = 4: six additions instead of twenty): every
+// lane returns the sum of quantity lane * N / 32
+template <int N>
+__device__ __forceinline__ double warp_sum(double (&v)[N])
 {
     const int lane = threadIdx.x & 31;
     int m = 16;
@@ -96,69 +78,27 @@ __device__ __forceinline__ A1 warp_sum(A1 (&v)[N])
         const bool up = (lane & m) != 0;
 #pragma unroll
         for (int k = 0; k < n; ++k) {
-            A1 x = up ? v[n + k] : v[k];
-            x.join((up ? v[k] : v[n + k]).from(m));
-            v[k] = x;
+            const double x = up ? v[n + k] : v[k];
+            v[k] = x + __shfl_xor_sync(0xffffffffu, up ? v[k] : v[n + k], m);
         }
     }
-    for (; m >= 1; m >>= 1) v[0].join(v[0].from(m));
+    for (; m >= 1; m >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], m);
     return v[0];
 }
 
-// the scalars of the recurrences in the accuracy of the sums: double-float
-// for single, double for double (FP64 instructions depend on one another at
-// an order of magnitude more latency than FP32 ones)
-template <class T>
-struct Scalar;
-template <>
-struct Scalar<float> {
-    typedef df R;
-    static __device__ __forceinline__ df get(const Acc<float>& a) { return df_norm(df(a.h, a.l)); }
-    static __device__ __forceinline__ float round(df a) { return a.hi + a.lo; }
-    // a / b, b scaled to [1, 2) by its exponent
-    static __device__ __forceinline__ cx<df> div(cx<df> a, cx<df> b)
-    {
-        const float m = fmaxf(fabsf(b.re.hi), fabsf(b.im.hi));
-        const unsigned e = (__float_as_uint(m) >> 23) & 0xffu;
-        const float sc = __uint_as_float((e >= 253u ? 1u : 254u - e) << 23);
-        const cx<df> bs = mk(df(b.re.hi * sc, b.re.lo * sc), df(b.im.hi * sc, b.im.lo * sc));
-        const cx<df> as = mk(df(a.re.hi * sc, a.re.lo * sc), df(a.im.hi * sc, a.im.lo * sc));
-        const df d = df_norm(bs.re * bs.re + bs.im * bs.im);
-        const cx<df> n = cjmul(bs, as);
-        const float inv = __fdividef(1.0f, d.hi);
-        return mk(quot(df_norm(n.re), d, inv), quot(df_norm(n.im), d, inv));
-    }
-    // n / d, inv an approximation of 1 / d: the first quotient's remainder is
-    // one FMA (exact) and the low parts, and gives the second
-    static __device__ __forceinline__ df quot(df n, df d, float inv)
-    {
-        const float q = n.hi * inv;
-        const float r = fmaf(-q, d.hi, n.hi) + (n.lo - q * d.lo);
-        return df_norm(df(q, r * inv));
-    }
-};
-template <>
-struct Scalar<double> {
-    typedef double R;
-    static __device__ __forceinline__ double get(const Acc<double>& a) { return a.h; }
-    static __device__ __forceinline__ double round(double a) { return a; }
-    static __device__ __forceinline__ cx<double> div(cx<double> a, cx<double> b)
-    {
-        const double d = 1.0 / (b.re * b.re + b.im * b.im);
-        return d * cjmul(b, a);
-    }
-};
-template <class T>
-__device__ __forceinline__ cx<T> sround(cx<typename Scalar<T>::R> a)
+// the scalars of the recurrences, in double; the vectors take them rounded to
+// the storage arithmetic
+__device__ __forceinline__ cx<double> cdiv(cx<double> a, cx<double> b)
 {
-    return mk(Scalar<T>::round(a.re), Scalar<T>::round(a.im));
+    const double d = 1.0 / (b.re * b.re + b.im * b.im);
+    return d * cjmul(b, a);
 }
-template <class R>
-__device__ __forceinline__ R from_round(float x) { return df(x, 0.f); }
-template <class R>
-__device__ __forceinline__ R from_round(double x) { return x; }
 template <class T>
-__device__ __forceinline__ bool fin2(cx<T> a) { return isfinite(a.re) && isfinite(a.im); }
+__device__ __forceinline__ cx<T> sround(cx<double> a)
+{
+    return mk((T)a.re, (T)a.im);
+}
+__device__ __forceinline__ bool fin2(cx<double> a) { return isfinite(a.re) && isfinite(a.im); }
 
 // ---------------------------------------------------------------------------
 // barrier of the CTAs of one group (bounded, as in k_solve) and the sums
@@ -204,24 +144,23 @@ __device__ __noinline__ bool group_sync(const SolveArgs& A, Group& G)
 // f receives the group's sums of the N quantities v on thread 0.  The CTAs'
 // partials lie quantity by quantity: warp k adds those of quantity k, four
 // loads in flight per lane.
-template <int NW, int N, class A1, class F>
-__device__ __noinline__ bool group_reduce(const SolveArgs& A, Group& G, A1 (&v)[N], F f)
+template <int NW, int N, class F>
+__device__ __noinline__ bool group_reduce(const SolveArgs& A, Group& G, double (&v)[N], F f)
 {
-    static_assert(sizeof(A1) == 8, "partial sums travel as 8-byte words");
-    static_assert(N <= NW, "one warp per quantity");
-    __shared__ A1 sh[N][NW], tot[N];
+    static_assert(N <= NW && N <= SPLIT_NQ, "one warp per quantity");
+    __shared__ double sh[N][NW], tot[N];
     __shared__ int s_ok;
     constexpr int LQ = 32 / N;  // lanes per quantity
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     {
-        const A1 x = warp_sum<N>(v);
+        const double x = warp_sum<N>(v);
         if (lane % LQ == 0) sh[lane / LQ][w] = x;
     }
     __syncthreads();
     ++G.epoch;
     if (G.cps == 1) {
         if (w < N) {
-            A1 q[1] = {A1::zero()};
+            double q[1] = {0.0};
             if (lane < NW) q[0] = sh[w][lane];
             q[0] = warp_sum<1>(q);
             if (lane == 0) tot[w] = q[0];
@@ -234,22 +173,23 @@ __device__ __noinline__ bool group_reduce(const SolveArgs& A, Group& G, A1 (&v)[
     double* part = A.part + ((size_t)G.rb * gridDim.x + (size_t)G.grp * G.cps) * SPLIT_NQ;
     if (w == 0) {
         // lane LQ k + j adds every LQ-th warp's sum of quantity k
-        A1 x = A1::zero();
+        double x = 0.0;
 #pragma unroll
         for (int j = 0; j < (NW + LQ - 1) / LQ; ++j) {
             const int i = lane % LQ + j * LQ;
-            if (i < NW) x.join(sh[lane / LQ][i]);
+            if (i < NW) x += sh[lane / LQ][i];
         }
 #pragma unroll
-        for (int m = LQ / 2; m >= 1; m >>= 1) x.join(x.from(m));
-        if (lane % LQ == 0) part[(size_t)(lane / LQ) * G.cps + G.cin] = x.bits();
+        for (int m = LQ / 2; m >= 1; m >>= 1)
+            if (m < NW) x += __shfl_xor_sync(0xffffffffu, x, m);
+        if (lane % LQ == 0) part[(size_t)(lane / LQ) * G.cps + G.cin] = x;
         __syncwarp();
         if (lane == 0) s_ok = group_wait(A, G);
     }
     __syncthreads();
     if (w < N) {
         const double* p = part + (size_t)w * G.cps;
-        A1 q[1] = {A1::zero()};
+        double q[1] = {0.0};
         for (int c = lane; c < G.cps; c += 128) {
             double u[4];
 #pragma unroll
@@ -257,7 +197,7 @@ __device__ __noinline__ bool group_reduce(const SolveArgs& A, Group& G, A1 (&v)[
                 if (c + 32 * k < G.cps) u[k] = __ldcg(p + c + 32 * k);
 #pragma unroll
             for (int k = 0; k < 4; ++k)
-                if (c + 32 * k < G.cps) q[0].join(A1::of(u[k]));
+                if (c + 32 * k < G.cps) q[0] += u[k];
         }
         q[0] = warp_sum<1>(q);
         if (lane == 0) tot[w] = q[0];
@@ -306,8 +246,13 @@ __device__ __forceinline__ double2 waxpy(cx<double> a, double2 x, double2 y)
 {
     return make_double2(y.x + a.re * x.x - a.im * x.y, y.y + a.re * x.y + a.im * x.x);
 }
-__device__ __forceinline__ void wnorm(float4 a, Acc<float>& n) { n.add(a.x * a.x + a.y * a.y + a.z * a.z + a.w * a.w); }
-__device__ __forceinline__ void wnorm(double2 a, Acc<double>& n) { n.add(a.x * a.x + a.y * a.y); }
+// |a|^2, Re <a, b> and Im <a, b> of a word
+__device__ __forceinline__ float wnorm(float4 a) { return a.x * a.x + a.y * a.y + a.z * a.z + a.w * a.w; }
+__device__ __forceinline__ double wnorm(double2 a) { return a.x * a.x + a.y * a.y; }
+__device__ __forceinline__ float wdot_re(float4 a, float4 b) { return a.x * b.x + a.y * b.y + a.z * b.z + a.w * b.w; }
+__device__ __forceinline__ float wdot_im(float4 a, float4 b) { return a.x * b.y - a.y * b.x + a.z * b.w - a.w * b.z; }
+__device__ __forceinline__ double wdot_re(double2 a, double2 b) { return a.x * b.x + a.y * b.y; }
+__device__ __forceinline__ double wdot_im(double2 a, double2 b) { return a.x * b.y - a.y * b.x; }
 
 __device__ __forceinline__ void put(Spinor<float>& s, int k, float4 w)
 {
@@ -677,15 +622,15 @@ __device__ __forceinline__ void for_words(const SolveArgs& A, int warp, int lane
 template <class W>
 struct W2 { W x, y; };
 template <class W>
-struct W5 { W s, t, v, p, e; };
+struct W3 { W r, v, p; };
+template <class W>
+struct W5 { W s, t, p, e, rh; };
 
 template <int P, int LPS, int BS, int MINB, int METHOD>
 __global__ void __launch_bounds__(BS, MINB) k_split(const __grid_constant__ SolveArgs A)
 {
     typedef typename Real<P>::T T;
     typedef typename Word<P>::W W;
-    typedef Scalar<T> SC;
-    typedef typename SC::R R;
     constexpr int NWORD = Word<P>::N;
     constexpr int NW = BS / 32, SG = NW / LPS;
     // the residual sweeps read x, as df pairs (xs) around a single-precision
@@ -697,12 +642,12 @@ __global__ void __launch_bounds__(BS, MINB) k_split(const __grid_constant__ Solv
     extern __shared__ __align__(16) unsigned char split_dyn[];
     __shared__ struct {
         double bn2, rn2, itol2;
-        cx<R> rho, d;
-        cx<T> alpha, omega, beta;
-        T best;  // smallest inner residual so far, and the iterations since
+        cx<double> rho, d, om;
+        cx<T> alpha, omega, beta;  // rounded to the storage arithmetic
+        double best;               // smallest inner residual so far, and the iterations since
         int since, idone, it, itc;
     } S;
-    __shared__ Acc<T> sums[METHOD == SOLVER_BICGSTAB ? 8 : 1][BS];
+    __shared__ double sums[METHOD == SOLVER_BICGSTAB ? 3 : 1][BS];
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     Group G;
@@ -753,7 +698,7 @@ __global__ void __launch_bounds__(BS, MINB) k_split(const __grid_constant__ Solv
 
         // ---- |b|^2; from x = 0: r64 = b
         {
-            Acc<double> q[1] = {Acc<double>::zero()};
+            double q[1] = {0.0};
             for_words<2, 12, NW>(
                 WORDS, [&](int i, int c) { return __ldg(bb + DW(i, c)); },
                 [&](int i, int c, double2 v) {
@@ -764,10 +709,10 @@ __global__ void __launch_bounds__(BS, MINB) k_split(const __grid_constant__ Solv
                         r6[a] = v;
                         xx[a] = make_double2(0.0, 0.0);
                     }
-                    q[0].add(v.x * v.x + v.y * v.y);
+                    q[0] += v.x * v.x + v.y * v.y;
                 });
-            if (!group_reduce<NW, 1>(A, G, q, [&](const Acc<double>(&n)[1]) {
-                    S.bn2 = S.rn2 = n[0].h;
+            if (!group_reduce<NW, 1>(A, G, q, [&](const double(&n)[1]) {
+                    S.bn2 = S.rn2 = n[0];
                     S.it = 0;
                 }))
                 return;
@@ -795,7 +740,7 @@ __global__ void __launch_bounds__(BS, MINB) k_split(const __grid_constant__ Solv
                     for (int s = 0; s < 4; ++s) store_comp<PT>(A.t64, 3 * s + r_, i, h[s]);
                 }
                 SYNC_OR_RETURN;
-                Acc<double> q[1] = {Acc<double>::zero()};
+                double q[1] = {0.0};
                 FOR_ITEMS
                 {
                     cx<TR> h[4];
@@ -807,10 +752,10 @@ __global__ void __launch_bounds__(BS, MINB) k_split(const __grid_constant__ Solv
                         const double re = b2.x - A.diag * x2.x + A.k2 * as_double(h[s].re);
                         const double im = b2.y - A.diag * x2.y + A.k2 * as_double(h[s].im);
                         r6[o] = make_double2(re, im);
-                        q[0].add(re * re + im * im);
+                        q[0] += re * re + im * im;
                     }
                 }
-                if (!group_reduce<NW, 1>(A, G, q, [&](const Acc<double>(&n)[1]) { S.rn2 = n[0].h; })) return;
+                if (!group_reduce<NW, 1>(A, G, q, [&](const double(&n)[1]) { S.rn2 = n[0]; })) return;
             }
             {
                 // every CTA of the group takes the same decision from the same sums
@@ -826,7 +771,7 @@ __global__ void __launch_bounds__(BS, MINB) k_split(const __grid_constant__ Solv
             ++outer;
             // ---- inner start: r = rh = p = r64 / |r64|, e = 0 (series: r = p)
             {
-                Acc<T> q[1] = {Acc<T>::zero()};
+                Local<T> loc = Local<T>::zero();
                 const double sc = 1.0 / sqrt(S.rn2);
                 for_words<2, NWORD, NW>(
                     WORDS,
@@ -849,11 +794,12 @@ __global__ void __launch_bounds__(BS, MINB) k_split(const __grid_constant__ Solv
                             V_(rh)[a] = w;
                             V_(e)[a] = wzero(W());
                         }
-                        wnorm(w, q[0]);
+                        loc.add(wnorm(w));
                     });
-                if (!group_reduce<NW, 1>(A, G, q, [&](const Acc<T>(&n)[1]) {
-                        S.rho = mk(SC::get(n[0]), R(0));
-                        S.best = SC::round(SC::get(n[0]));
+                double q[1] = {loc.value()};
+                if (!group_reduce<NW, 1>(A, G, q, [&](const double(&n)[1]) {
+                        S.rho = mk(n[0], 0.0);
+                        S.best = n[0];
                         S.since = 0;
                         S.idone = 0;
                         S.itc = 0;
@@ -870,7 +816,7 @@ __global__ void __launch_bounds__(BS, MINB) k_split(const __grid_constant__ Solv
                 const T k2 = (T)A.k2, dinv = (T)(1.0 / A.diag);
                 for (;;) {
                     const bool chk = (S.itc & 1) || S.itc + 1 >= A.max_inner || S.it + 1 >= A.max_iter;
-                    Acc<T> q[1] = {Acc<T>::zero()};
+                    double q[1] = {0.0};
 #pragma unroll 1
                     for (int par = 1; par >= 0; --par) {
                         const W* in = par ? V_(p) : V_(tmp);
@@ -893,7 +839,7 @@ __global__ void __launch_bounds__(BS, MINB) k_split(const __grid_constant__ Solv
                                         pp[k] = o[k] - pp[k];
                                     }
                                     store_part<NC>(V_(p) + at, d, o);
-                                    if (chk) q[0].add(pnorm<NC>(pp));
+                                    if (chk) q[0] += (double)pnorm<NC>(pp);
                                 }
                             }
                         }
@@ -908,10 +854,10 @@ __global__ void __launch_bounds__(BS, MINB) k_split(const __grid_constant__ Solv
                         __syncthreads();
                         continue;
                     }
-                    if (!group_reduce<NW, 1>(A, G, q, [&](const Acc<T>(&n)[1]) {
+                    if (!group_reduce<NW, 1>(A, G, q, [&](const double(&n)[1]) {
                             S.it += 1;
                             S.itc += 1;
-                            const double res2 = A.diag * A.diag * (double)SC::round(SC::get(n[0]));
+                            const double res2 = A.diag * A.diag * n[0];
                             if (!(res2 > S.itol2) || S.itc >= A.max_inner || S.it >= A.max_iter) S.idone = 1;
                             // a series that grows cannot converge: reported as not converged
                             if (!isfinite(res2) || (S.itc >= 16 && res2 > 1e6)) {
@@ -923,21 +869,22 @@ __global__ void __launch_bounds__(BS, MINB) k_split(const __grid_constant__ Solv
                     if (S.idone) break;
                 }
             } else {
-                // ---- BiCGstab, six barriers an iteration, two of them reducing:
+                // ---- BiCGstab, seven barriers an iteration, three of them reducing:
                 //   0  tmp = H_oe p        1  v = A p, <rh, v> -> alpha      s = r - alpha v
-                //   2  tmp = H_oe s        3  t = A s and the sums of omega, beta
-                //   e += alpha p + omega s, r = s - omega t, p = r + beta (p - omega v)
-                // <rh, r> and |r|^2 of the new residual follow from the sums of step
-                // 3, so beta is known before r is formed.  One copy of the
-                // hopping code serves all four sweeps: it has to fit the
-                // instruction cache.
+                //   2  tmp = H_oe s        3  t = A s, <t, s>, |t|^2 -> omega
+                //   e += alpha p + omega s, r = s - omega t, <rh, r>, |r|^2 -> beta
+                //   p = r + beta (p - omega v)
+                // (<rh, r> and |r|^2 also follow from sums over s and t, without the
+                // last reduction, but lose what one step reduces the residual by.)
+                // One copy of the hopping code serves all four sweeps: it has to
+                // fit the instruction cache.
                 const T k2 = (T)A.k2, dg = (T)A.diag;
                 bool stop = false;
                 for (;;) {
 #pragma unroll 1
                     for (int ph = 0; ph < 4; ++ph) {
                         const W* in = ph == 0 ? V_(p) : ph == 2 ? V_(r) : V_(tmp);
-                        // the thread's sums wait in shared memory: sixteen registers less in the hops
+                        // the thread's sums wait in shared memory: six registers less in the hops
                         bool some = false;
                         FOR_GROUPS
                         {
@@ -951,46 +898,33 @@ __global__ void __launch_bounds__(BS, MINB) k_split(const __grid_constant__ Solv
                                 } else {
                                     cx<T> y[NC], z[NC];
                                     load_part<NC>((ph == 1 ? V_(p) : V_(r)) + at, d, y);
-                                    load_part<NC>(V_(rh) + at, d, z);
 #pragma unroll
                                     for (int k = 0; k < NC; ++k) o[k] = dg * y[k] - k2 * o[k];
                                     store_part<NC>((ph == 1 ? V_(v) : V_(t)) + at, d, o);
-                                    T n[8];
-                                    pdot<NC>(z, o, n[0], n[1]);
-                                    if (ph == 3) {
-                                        pdot<NC>(z, y, n[2], n[3]);
-                                        pdot<NC>(o, y, n[4], n[5]);
-                                        n[6] = pnorm<NC>(o);
-                                        n[7] = pnorm<NC>(y);
+                                    T n[3];
+                                    if (ph == 1) {
+                                        load_part<NC>(V_(rh) + at, d, z);
+                                        pdot<NC>(z, o, n[0], n[1]);
+                                    } else {
+                                        pdot<NC>(o, y, n[0], n[1]);
+                                        n[2] = pnorm<NC>(o);
                                     }
 #pragma unroll
-                                    for (int k = 0; k < 8; ++k)
-                                        if (k < 2 || ph == 3) {
-                                            Acc<T> s = Acc<T>::zero();
-                                            if (some) s = sums[k][tid];
-                                            s.add(n[k]);
-                                            sums[k][tid] = s;
-                                        }
+                                    for (int k = 0; k < 3; ++k)
+                                        if (k < 2 || ph == 3) sums[k][tid] = some ? sums[k][tid] + (double)n[k] : (double)n[k];
                                     some = true;
                                 }
                             }
                         }
-                        Acc<T> q[8];
-#pragma unroll
-                        for (int k = 0; k < 8; ++k) {
-                            q[k] = Acc<T>::zero();
-                            if (some && (k < 2 || ph == 3)) q[k] = sums[k][tid];
-                        }
                         if (!(ph & 1)) {
                             SYNC_OR_RETURN;
                         } else if (ph == 1) {
-                            Acc<T> q2[4] = {q[0], q[1], Acc<T>::zero(), Acc<T>::zero()};
-                            if (!group_reduce<NW, 4>(A, G, q2, [&](const Acc<T>(&n)[4]) {
-                                    const cx<R> dn = mk(SC::get(n[0]), SC::get(n[1]));
-                                    const cx<T> d0 = sround<T>(dn), al = sround<T>(SC::div(S.rho, dn));
+                            double q[2] = {some ? sums[0][tid] : 0.0, some ? sums[1][tid] : 0.0};
+                            if (!group_reduce<NW, 2>(A, G, q, [&](const double(&n)[2]) {
+                                    const cx<double> dn = mk(n[0], n[1]), al = cdiv(S.rho, dn);
                                     S.d = dn;
-                                    if (!fin2(al) || (d0.re == T(0) && d0.im == T(0))) S.idone = 1;
-                                    else S.alpha = al;
+                                    if (!fin2(al) || (n[0] == 0.0 && n[1] == 0.0)) S.idone = 1;
+                                    else S.alpha = sround<T>(al);
                                 }))
                                 return;
                             if (S.idone) {  // the sums gave no step
@@ -1003,73 +937,81 @@ __global__ void __launch_bounds__(BS, MINB) k_split(const __grid_constant__ Solv
                                 [&](int i, int k, W2<W> w) { V_(r)[TW(i, k)] = waxpy(mal, w.y, w.x); });
                             SYNC_OR_RETURN;
                         } else {
-                            if (!group_reduce<NW, 8>(A, G, q, [&](const Acc<T>(&n)[8]) {
-                                    const cx<R> rt = mk(SC::get(n[0]), SC::get(n[1])), rs = mk(SC::get(n[2]), SC::get(n[3]));
-                                    const cx<R> ts = mk(SC::get(n[4]), SC::get(n[5]));
-                                    const R tt = SC::get(n[6]), ss = SC::get(n[7]);
-                                    cx<T> om = sround<T>(SC::div(ts, mk(tt, R(0))));
-                                    if (!(SC::round(tt) > T(0)) || !fin2(om)) {
-                                        om = mk(T(0), T(0));
+                            double q[4] = {some ? sums[0][tid] : 0.0, some ? sums[1][tid] : 0.0, some ? sums[2][tid] : 0.0, 0.0};
+                            if (!group_reduce<NW, 4>(A, G, q, [&](const double(&n)[4]) {
+                                    const double inv = 1.0 / n[2];
+                                    cx<double> om = mk(n[0] * inv, n[1] * inv);
+                                    if (!(n[2] > 0.0) || !fin2(om)) {
+                                        om = mk(0.0, 0.0);
                                         S.idone = 1;  // keep alpha p, stop afterwards
                                     }
-                                    S.omega = om;
-                                    S.it += 1;
-                                    S.itc += 1;
-                                    const cx<R> omr = mk(from_round<R>(om.re), from_round<R>(om.im));
-                                    const cx<R> rn = rs - omr * rt;
-                                    // |s - omega t|^2
-                                    const R two = from_round<R>(T(2));
-                                    const R rr = ss - two * (omr.re * ts.re + omr.im * ts.im) +
-                                                 (omr.re * omr.re + omr.im * omr.im) * tt;
-                                    const T rf = SC::round(rr);
-                                    // far above its start (1) the recurrence has diverged: keep the
-                                    // correction so far, the outer cycle recomputes the residual
-                                    if (S.itc >= A.max_inner || S.it >= A.max_iter || !((double)rf > S.itol2) ||
-                                        !fin2(sround<T>(rn)) || rf > T(1e8))
-                                        S.idone = 1;
-                                    // a residual that has stalled: restarted from the true one
-                                    if (rf < S.best) {
-                                        S.best = rf;
-                                        S.since = 0;
-                                    } else if (++S.since >= STALL) {
-                                        S.idone = 1;
-                                    }
-                                    if (!S.idone) {
-                                        // beta = (rn / rho) (alpha / omega) with alpha = rho / d
-                                        const cx<T> be = sround<T>(SC::div(rn, S.d * omr));
-                                        if (!fin2(be)) S.idone = 1;
-                                        S.beta = be;
-                                        S.rho = rn;
-                                    }
+                                    S.om = om;
+                                    S.omega = sround<T>(om);
                                 }))
                                 return;
                         }
                     }
                     if (stop) break;
+                    constexpr int B = P == PREC32 ? 3 : 2;
                     {
-                        const cx<T> al = S.alpha, om = S.omega, be = S.beta;
-                        const bool more = !S.idone;
-                        constexpr int B = P == PREC32 ? 3 : 2;
+                        const cx<T> al = S.alpha, om = S.omega;
+                        Local<T> l0 = Local<T>::zero(), l1 = l0, l2 = l0;
                         for_words<B, NWORD, NW>(
                             WORDS,
                             [&](int i, int k) {
                                 const size_t a = TW(i, k);
-                                return W5<W>{V_(r)[a], V_(t)[a], V_(v)[a], V_(p)[a], V_(e)[a]};
+                                return W5<W>{V_(r)[a], V_(t)[a], V_(p)[a], V_(e)[a], V_(rh)[a]};
                             },
                             [&](int i, int k, W5<W> w) {
                                 const size_t a = TW(i, k);
                                 V_(e)[a] = waxpy(om, w.s, waxpy(al, w.p, w.e));
-                                if (more) {
-                                    const W rr = waxpy(-om, w.t, w.s);
-                                    V_(r)[a] = rr;
-                                    V_(p)[a] = waxpy(be, waxpy(-om, w.v, w.p), rr);
-                                }
+                                const W rr = waxpy(-om, w.t, w.s);
+                                V_(r)[a] = rr;
+                                l0.add(wdot_re(w.rh, rr));
+                                l1.add(wdot_im(w.rh, rr));
+                                l2.add(wnorm(rr));
                             });
+                        double q[4] = {l0.value(), l1.value(), l2.value(), 0.0};
+                        if (!group_reduce<NW, 4>(A, G, q, [&](const double(&n)[4]) {
+                                S.it += 1;
+                                S.itc += 1;
+                                const cx<double> rn = mk(n[0], n[1]);
+                                const double rr = n[2];
+                                // far above its start (1) the recurrence has diverged: keep the
+                                // correction so far, the outer cycle recomputes the residual
+                                if (S.itc >= A.max_inner || S.it >= A.max_iter || !(rr > S.itol2) || !fin2(rn) ||
+                                    rr > 1e8)
+                                    S.idone = 1;
+                                // a residual that has stalled: restarted from the true one
+                                if (rr < S.best) {
+                                    S.best = rr;
+                                    S.since = 0;
+                                } else if (++S.since >= STALL) {
+                                    S.idone = 1;
+                                }
+                                if (!S.idone) {
+                                    // beta = (rn / rho) (alpha / omega) with alpha = rho / d
+                                    const cx<double> be = cdiv(rn, S.d * S.om);
+                                    if (!fin2(be)) S.idone = 1;
+                                    S.beta = sround<T>(be);
+                                    S.rho = rn;
+                                }
+                            }))
+                            return;
                     }
                     if (S.idone) break;
+                    {
+                        const cx<T> om = S.omega, be = S.beta;
+                        for_words<B, NWORD, NW>(
+                            WORDS,
+                            [&](int i, int k) {
+                                const size_t a = TW(i, k);
+                                return W3<W>{V_(r)[a], V_(v)[a], V_(p)[a]};
+                            },
+                            [&](int i, int k, W3<W> w) { V_(p)[TW(i, k)] = waxpy(be, waxpy(-om, w.v, w.p), w.r); });
+                    }
                     SYNC_OR_RETURN;
                 }
-                SYNC_OR_RETURN;
             }
 
             // ---- x += |r64| e
