@@ -33,6 +33,7 @@ struct SolveArgs {
     SpinorF r, rh, p, v, s, t;  // inner precision, parity 0
     SpinorF tmp;        // inner precision, parity 1
     SpinorF e;          // inner solution (single; double for the double solver)
+    SpinorF eb;         // its best iterate (lqcd_split.cu)
     double tol, inner_tol;
     int max_iter, max_outer, max_inner;
     double* part;       // double-buffered partial sums of every CTA

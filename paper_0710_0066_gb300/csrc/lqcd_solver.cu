@@ -2050,6 +2050,8 @@ int eo_solve(lqcd_ctx* h, int mode, int colour, int prec, double kappa, double2*
     A.t = inner_view(w->vec[5], prec, g.Vh);
     A.tmp = inner_view(w->vec[6], prec, g.Vh);
     A.e = inner_view(w->vec[7], prec == PREC64 ? PREC64 : PREC32, g.Vh);
+    // (a double solve leaves s unused, a single one half of every buffer)
+    A.eb = prec == PREC64 ? A.s : inner_view(w->vec[7] + (size_t)6 * ((g.Vh + 31) & ~31), PREC32, g.Vh);
     if (sap) {
         LQ_TRY(solver_sap_alloc(h));
         SpinorF* fv[Work::NSAP] = {A.fr, A.frh, A.fp, A.fv, A.fs, A.ft, A.fzp, A.fzs, A.fw1, A.fw2, A.fy};
@@ -2067,7 +2069,8 @@ int eo_solve(lqcd_ctx* h, int mode, int colour, int prec, double kappa, double2*
     // early and leave more of the reduction to the double outer cycles)
     A.inner_tol = prec == PREC64 ? 0.0 : prec == PREC32 ? 1e-5 : prec == PREC16 ? 2e-3 : 3e-2;
     A.max_iter = max_iter;
-    A.max_outer = prec == PRECBF ? 80 : 40;
+    // (the Schwarz solve in double restarts only after a breakdown)
+    A.max_outer = prec == PRECBF ? 80 : prec == PREC64 && sap ? 8 : 40;
     A.max_inner = prec == PREC64 ? max_iter : prec == PREC32 ? 4000 : prec == PREC16 ? 600 : 200;
     A.part = w->part;
     A.bar = w->bar;

@@ -98,7 +98,8 @@ __device__ __forceinline__ cx<T> sround(cx<double> a)
 {
     return mk((T)a.re, (T)a.im);
 }
-__device__ __forceinline__ bool fin2(cx<double> a) { return isfinite(a.re) && isfinite(a.im); }
+template <class T>
+__device__ __forceinline__ bool fin2(cx<T> a) { return isfinite(a.re) && isfinite(a.im); }
 
 // ---------------------------------------------------------------------------
 // barrier of the CTAs of one group (bounded, as in k_solve) and the sums
@@ -587,12 +588,21 @@ __device__ __forceinline__ int group_site(const SolveArgs& A, int g)
     return (((((x0 << (A.nt[0] + A.lt[1])) + x1) << A.nt[1]) + tq) << (A.lt[2] + 5)) + (q << 5);
 }
 
-// BiCGstab iterations without a new smallest residual after which the inner
-// solve ends and the outer cycle restarts it from the true residual.  A
-// system near its critical point (8x4^3, kappa = 0.15 on a smooth field, in
-// double): 1400-2300 iterations in 5 cycles with a restart after 100,
-// 3000-4000 after 300, without one 2900 to no convergence, as rounding has it.
+// Near a critical point the BiCGstab recurrence stalls: its residual stops
+// falling for thousands of iterations, or for good, as rounding has it.  An
+// inner solve that has gone `window` iterations without a new smallest |r|^2
+// ends, and the outer cycle restarts it from the true residual of its best
+// iterate (kept whenever |r| has halved), so a restart never adds a correction
+// that is worse than its start.  It ends only where it has gained something,
+// and where a cycle ended so has gained less than 1 / 0.3 the window doubles: a
+// plateau that is longer than the window is waited out at the second or third
+// try, and twelve decades take at most 23 such cycles and 7 doublings, fewer
+// than the outer cycles allowed.  Iterations to 1e-12, four sources at 8x4^3
+// near criticality (kappa = 0.15): double 2200-3100, single storage 3800-4700;
+// restarted from the current iterate after a fixed 200: 2600-3900 and
+// 6200-8600; not restarted: 11 600 to no convergence, and no convergence.
 constexpr int STALL = 200;
+constexpr double STALL_GAIN = 0.3;
 
 // (site, word) items of the element-wise phases, B of them at a time so that
 // their loads are in flight together: act(site, word, load(site, word)).  An
@@ -644,8 +654,11 @@ __global__ void __launch_bounds__(BS, MINB) k_split(const __grid_constant__ Solv
         double bn2, rn2, itol2;
         cx<double> rho, d, om;
         cx<T> alpha, omega, beta;  // rounded to the storage arithmetic
-        double best;               // smallest inner residual so far, and the iterations since
-        int since, idone, it, itc;
+        // |r|^2: at the inner start, now, the smallest so far, that of the iterate
+        // kept in A.eb; iterations since the smallest
+        double start, rr, best, kept;
+        int since, window, stalled, keep, use_kept;
+        int idone, it, itc;
     } S;
     __shared__ double sums[METHOD == SOLVER_BICGSTAB ? 3 : 1][BS];
 
@@ -714,6 +727,8 @@ __global__ void __launch_bounds__(BS, MINB) k_split(const __grid_constant__ Solv
             if (!group_reduce<NW, 1>(A, G, q, [&](const double(&n)[1]) {
                     S.bn2 = S.rn2 = n[0];
                     S.it = 0;
+                    S.window = STALL;
+                    S.stalled = 0;
                 }))
                 return;
         }
@@ -755,7 +770,12 @@ __global__ void __launch_bounds__(BS, MINB) k_split(const __grid_constant__ Solv
                         q[0] += re * re + im * im;
                     }
                 }
-                if (!group_reduce<NW, 1>(A, G, q, [&](const double(&n)[1]) { S.rn2 = n[0]; })) return;
+                if (!group_reduce<NW, 1>(A, G, q, [&](const double(&n)[1]) {
+                        // (S.rn2: the residual that the last inner solve started from)
+                        if (S.stalled && !(n[0] <= STALL_GAIN * STALL_GAIN * S.rn2)) S.window *= 2;
+                        S.stalled = 0;
+                        S.rn2 = n[0];
+                    })) return;
             }
             {
                 // every CTA of the group takes the same decision from the same sums
@@ -799,8 +819,8 @@ __global__ void __launch_bounds__(BS, MINB) k_split(const __grid_constant__ Solv
                 double q[1] = {loc.value()};
                 if (!group_reduce<NW, 1>(A, G, q, [&](const double(&n)[1]) {
                         S.rho = mk(n[0], 0.0);
-                        S.best = n[0];
-                        S.since = 0;
+                        S.start = S.rr = S.best = S.kept = n[0];
+                        S.since = S.keep = S.use_kept = 0;
                         S.idone = 0;
                         S.itc = 0;
                         const double need = 0.5 * A.tol * sqrt(S.bn2 / fmax(S.rn2, 1e-300));
@@ -921,10 +941,15 @@ __global__ void __launch_bounds__(BS, MINB) k_split(const __grid_constant__ Solv
                         } else if (ph == 1) {
                             double q[2] = {some ? sums[0][tid] : 0.0, some ? sums[1][tid] : 0.0};
                             if (!group_reduce<NW, 2>(A, G, q, [&](const double(&n)[2]) {
-                                    const cx<double> dn = mk(n[0], n[1]), al = cdiv(S.rho, dn);
+                                    const cx<double> dn = mk(n[0], n[1]);
+                                    const cx<T> al = sround<T>(cdiv(S.rho, dn));
                                     S.d = dn;
-                                    if (!fin2(al) || (n[0] == 0.0 && n[1] == 0.0)) S.idone = 1;
-                                    else S.alpha = sround<T>(al);
+                                    if (!fin2(al) || (n[0] == 0.0 && n[1] == 0.0)) {
+                                        S.idone = 1;
+                                        S.use_kept = S.kept < S.start && S.kept < S.rr;
+                                    } else {
+                                        S.alpha = al;
+                                    }
                                 }))
                                 return;
                             if (S.idone) {  // the sums gave no step
@@ -941,7 +966,7 @@ __global__ void __launch_bounds__(BS, MINB) k_split(const __grid_constant__ Solv
                             if (!group_reduce<NW, 4>(A, G, q, [&](const double(&n)[4]) {
                                     const double inv = 1.0 / n[2];
                                     cx<double> om = mk(n[0] * inv, n[1] * inv);
-                                    if (!(n[2] > 0.0) || !fin2(om)) {
+                                    if (!(n[2] > 0.0) || !fin2(sround<T>(om))) {
                                         om = mk(0.0, 0.0);
                                         S.idone = 1;  // keep alpha p, stop afterwards
                                     }
@@ -982,24 +1007,30 @@ __global__ void __launch_bounds__(BS, MINB) k_split(const __grid_constant__ Solv
                                 if (S.itc >= A.max_inner || S.it >= A.max_iter || !(rr > S.itol2) || !fin2(rn) ||
                                     rr > 1e8)
                                     S.idone = 1;
-                                // a residual that has stalled: restarted from the true one
+                                S.rr = rr;
+                                S.keep = rr < 0.25 * S.kept;
+                                if (S.keep) S.kept = rr;
                                 if (rr < S.best) {
                                     S.best = rr;
                                     S.since = 0;
-                                } else if (++S.since >= STALL) {
-                                    S.idone = 1;
+                                } else if (++S.since >= S.window && S.kept < S.start && !S.idone) {
+                                    S.idone = S.stalled = 1;
                                 }
                                 if (!S.idone) {
                                     // beta = (rn / rho) (alpha / omega) with alpha = rho / d
-                                    const cx<double> be = cdiv(rn, S.d * S.om);
-                                    if (!fin2(be)) S.idone = 1;
-                                    S.beta = sround<T>(be);
+                                    S.beta = sround<T>(cdiv(rn, S.d * S.om));
+                                    if (!fin2(S.beta)) S.idone = 1;
                                     S.rho = rn;
                                 }
+                                S.use_kept = S.kept < S.start && S.kept < rr;
                             }))
                             return;
                     }
                     if (S.idone) break;
+                    if (S.keep)
+                        for_words<B, NWORD, NW>(
+                            WORDS, [&](int i, int k) { return V_(e)[TW(i, k)]; },
+                            [&](int i, int k, W w) { V_(eb)[TW(i, k)] = w; });
                     {
                         const cx<T> om = S.omega, be = S.beta;
                         for_words<B, NWORD, NW>(
@@ -1017,7 +1048,7 @@ __global__ void __launch_bounds__(BS, MINB) k_split(const __grid_constant__ Solv
             // ---- x += |r64| e
             {
                 const double sc = sqrt(S.rn2);
-                const W* ev = METHOD == SOLVER_SERIES ? V_(p) : V_(e);
+                const W* ev = METHOD == SOLVER_SERIES ? V_(p) : S.use_kept ? V_(eb) : V_(e);
                 for_words<2, 12, NW>(
                     WORDS,
                     [&](int i, int c) {
