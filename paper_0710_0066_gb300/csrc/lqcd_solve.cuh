@@ -79,12 +79,14 @@ __device__ __forceinline__ unsigned ld_acquire(const unsigned* p)
 
 // lqcd_split.cu: the persistent solver of single- and double-precision inner
 // storage.  split_init sets its kernels' attributes and reads their occupancy
-// (gmax: the largest grid); split_plan picks the kernel for the systems of A
-// (spt: lqcd_set_solver_schedule) and sets cps, ngrp, chunk and the tiling.
+// (gmax: the largest grid) and the bytes of the L2; split_plan picks the
+// kernel for the systems of A (spt: lqcd_set_solver_schedule) and sets cps,
+// ngrp, chunk and the tiling.
 constexpr int SPLIT_NVAR = 6;
 struct SplitPlan {
     const void* fn;
     int grid, block, smem;
 };
-cudaError_t split_init(int num_sms, int occ[SPLIT_NVAR][2], int* gmax);
-SplitPlan split_plan(SolveArgs& A, int prec, int method, int spt, int num_sms, const int occ[SPLIT_NVAR][2]);
+cudaError_t split_init(int num_sms, int occ[SPLIT_NVAR][2], int* gmax, int* l2);
+SplitPlan split_plan(SolveArgs& A, int prec, int method, int spt, int num_sms, const int occ[SPLIT_NVAR][2],
+                     int l2);

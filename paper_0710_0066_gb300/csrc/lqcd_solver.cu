@@ -1771,6 +1771,7 @@ struct Work {
     double* h_resid = nullptr;
     int gmax[NPREC] = {0, 0, 0, 0};  // co-resident CTAs of k_solve per precision
     int split_occ[SPLIT_NVAR][2];    // CTAs per SM of the k_split variants
+    int l2 = 0;                      // bytes of the L2
     int cl_ok = 0;                   // the device runs k_series_cl's clusters
     // the Schwarz-preconditioned global solve: 11 full-lattice vectors, each
     // sized for a double full field (allocated on first use)
@@ -1860,7 +1861,7 @@ int solver_init(lqcd_ctx* h)
         gm = std::max(gm, w->gmax[k]);
     }
     int gsplit = 0;
-    LQ_CUDA(h, split_init(h->num_sms, w->split_occ, &gsplit));
+    LQ_CUDA(h, split_init(h->num_sms, w->split_occ, &gsplit, &w->l2));
     LQ_CUDA(h, cudaMalloc(&w->part, sizeof(double) * 2 * std::max(NQ * (size_t)gm, SPLIT_NQ * (size_t)gsplit)));
     LQ_CUDA(h, cudaMalloc(&w->bar, sizeof(unsigned) * BAR_STRIDE * NSYS_MAX));
     LQ_CUDA(h, cudaMalloc(&w->status, sizeof(int) * 4));
@@ -2114,7 +2115,7 @@ int eo_solve(lqcd_ctx* h, int mode, int colour, int prec, double kappa, double2*
                                       : (sap ? (const void*)k_solve<PRECBF, true> : (const void*)k_solve<PRECBF, false>);
     int grid = G, block = SBS;
     if (!clu && !sap && (prec == PREC64 || prec == PREC32)) {
-        const SplitPlan sp = split_plan(A, prec, method, spt, h->num_sms, w->split_occ);
+        const SplitPlan sp = split_plan(A, prec, method, spt, h->num_sms, w->split_occ, w->l2);
         fn = sp.fn;
         grid = sp.grid;
         block = sp.block;

@@ -1140,32 +1140,41 @@ int pick(int prec, int groups, int num_sms)
     return groups <= 16 * num_sms ? V_1 : V_1W;
 }
 
-// How many of the systems a launch works on at a time.  Vectors and links that
-// an iteration of all of them reads and writes again may not fit the 129 MB L2
-// (96 bytes a vector and site, 384 the site's links); half as many at a time
-// do, and the sweeps are bound by L2 traffic.  Systems of 32x24^3 in slabs of
-// 8 (170 MB), series: four at a time 8.02 ms, two 7.64.  Not below the number
-// of groups at which one CTA per SM is filled: one at a time 10.3 ms.
-int systems_at_once(const SolveArgs& A, int prec, int method, int num_sms)
+// How many of the systems a launch works on at a time.  What a series iteration
+// of all of them reads and writes again (three vectors of 96 bytes a site and
+// 384 of links) may not fit the L2; a part of the systems does, and the sweeps
+// are bound by L2 traffic.  Full waves only (a divisor of the number of systems;
+// an uneven last wave leaves SMs idle: eight systems of 32000 sites by three
+// 6.68 ms, by four 5.81, at once 6.41), each within three quarters of the L2 and
+// wide enough to fill the chip.  Measured (ms at 66 iterations, at once -> in
+// these waves): 8 x 30976 sites 6.34 -> 5.39, 8 x 55296 10.87 -> 10.54, 4 x 131072
+// 12.27 -> 11.51, 4 x 55296 5.26 -> 5.17 (122 iterations: 8.02 -> 7.64),
+// 8 x 131072 23.8 -> 23.3; with few iterations the waves' start and end weigh
+// more (38: 4 x 55296 3.83 -> 3.85, 8 x 131072 17.0 -> 17.4).  BiCGstab, seven
+// vectors, runs at once: waves 0-29 % slower (10 x 27648 5.07 ms, by four 6.5;
+// 4 x 46080 3.69, by two 3.92; the best of them, 8 x 30976 by four, 2 % faster).
+int systems_at_once(const SolveArgs& A, int prec, int method, int num_sms, int l2)
 {
-    constexpr double L2 = 129e6, FIT = 96e6;
-    const double set = (method == SOLVER_SERIES ? 4 * 96.0 + 384.0 : 6 * 96.0 + 384.0) * A.nsite;
-    if (prec != PREC32 || set * A.nsys <= L2) return A.nsys;
-    const int n = (int)(FIT / set);
-    if (n < 1) return A.nsys;
-    const int waves = (A.nsys + n - 1) / n, at = (A.nsys + waves - 1) / waves;
-    return (A.nsite + 31) / 32 * at >= 16 * num_sms ? at : A.nsys;
+    const double set = (3 * 96.0 + 384.0) * A.nsite;
+    if (prec != PREC32 || method != SOLVER_SERIES || set * A.nsys <= l2) return A.nsys;
+    int at = A.nsys;
+    while (at > 1 && (A.nsys % at != 0 || set * at > 0.75 * l2)) --at;
+    return set * at <= 0.75 * l2 && (A.nsite + 31) / 32 * at >= 20 * num_sms ? at : A.nsys;
 }
 
 }  // namespace
 
-cudaError_t split_init(int num_sms, int occ[SPLIT_NVAR][2], int* gmax)
+cudaError_t split_init(int num_sms, int occ[SPLIT_NVAR][2], int* gmax, int* l2)
 {
     *gmax = 0;
+    int dev;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(l2, cudaDevAttrL2CacheSize, dev);
+    if (e != cudaSuccess) return e;
     for (int k = 0; k < SPLIT_NVAR; ++k)
         for (int m = 0; m < 2; ++m) {
             const Variant& v = variants[k];
-            cudaError_t e = cudaFuncSetAttribute(v.fn[m], cudaFuncAttributeMaxDynamicSharedMemorySize, v.smem);
+            e = cudaFuncSetAttribute(v.fn[m], cudaFuncAttributeMaxDynamicSharedMemorySize, v.smem);
             if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[k][m], v.fn[m], v.bs, v.smem);
             if (e != cudaSuccess) return e;
             if (occ[k][m] < 1) return cudaErrorLaunchOutOfResources;
@@ -1174,10 +1183,11 @@ cudaError_t split_init(int num_sms, int occ[SPLIT_NVAR][2], int* gmax)
     return cudaSuccess;
 }
 
-SplitPlan split_plan(SolveArgs& A, int prec, int method, int spt, int num_sms, const int occ[SPLIT_NVAR][2])
+SplitPlan split_plan(SolveArgs& A, int prec, int method, int spt, int num_sms, const int occ[SPLIT_NVAR][2],
+                     int l2)
 {
     const int G = (A.nsite + 31) / 32;
-    A.ngrp = systems_at_once(A, prec, method, num_sms);
+    A.ngrp = systems_at_once(A, prec, method, num_sms, l2);
     const int k = pick(prec, G * A.ngrp, num_sms), m = method == SOLVER_SERIES ? 1 : 0;
     const Variant& v = variants[k];
     const int SG = v.bs / 32 / v.lps;  // groups a CTA holds side by side
