@@ -78,9 +78,9 @@ def thermalise_dynamical(lat, U, prm, ntraj, seed):
 
 PEAKS = os.path.join(ROOT, "MEASURED_PEAKS.json")
 
-# DRAM bytes per solver launch from the ncu capture summarised in
-# profiles/k_split_16x16x16x32_f32.md, valid only for the solver source
-# that was captured (bench.py reports null once the source differs)
+# DRAM bytes per solver launch from an ncu capture at 16^3x32 in single
+# precision, valid only for the solver source that was captured (bench.py
+# reports null once the source differs)
 SOLVER_SOURCES = ("lqcd_split.cu", "lqcd_solve.cuh", "lqcd_common.cuh", "lqcd_df.cuh")  # the sources k_split is built from
 SOLVER_TRAFFIC = dict(src_sha256="d361f8bf57e40fdc75a5514e4db0ebe94ea8c46190e0eda92521a7be04447471",
                       block_series=(346.314e6 + 147.963e6), block=(426.858e6 + 442.421e6),
@@ -103,7 +103,7 @@ def solver_traffic():
     return SOLVER_TRAFFIC["block_series"], {"batched_slab_solve_series": SOLVER_TRAFFIC["block_series"],
                                             "batched_slab_solve_bicgstab": SOLVER_TRAFFIC["block"],
                                             "global_solve_bicgstab": SOLVER_TRAFFIC["glob"],
-                                            "source": "profiles/k_split_16x16x16x32_f32.md"}
+                                            "source": "ncu dram__bytes, k_split F32 at 16^3x32"}
 
 
 def hbm_peak():

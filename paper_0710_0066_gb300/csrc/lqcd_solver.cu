@@ -12,8 +12,9 @@
 // lqcd_split.cu; k_solve here runs the half formats and every
 // Schwarz-preconditioned solve, k_series_cl the opt-in cluster form.
 // Each system is handled by its own group of CTAs (cps CTAs per system).
-// Reductions are per system, in double, in a fixed order (warp shuffles,
-// then the group's per-CTA partials summed in CTA order), so every CTA of a
+// Reductions are per system, in double (a site's term in the storage
+// arithmetic), in a fixed order (warp shuffles, then the group's per-CTA
+// partials summed in CTA order), so every CTA of a
 // group computes bitwise the same scalars and takes the same decisions.
 // The systems never wait for one another: a group meets only at its own
 // software barrier (one counter per system), loops until its own system has
@@ -1929,7 +1930,7 @@ void solver_site_bytes(int prec, int method, double* inner, double* outer, int n
     const double sp = prec == PREC64 ? 192.0 : prec == PREC32 ? 96.0 : prec == PREC16 ? 52.0 : 48.0;
     const double lk = prec == PREC64 ? 1152.0 : prec == PREC32 ? 384.0 : 192.0;
     const double se = prec == PREC64 ? 192.0 : 96.0;
-    // BiCGstab: 24 spinor passes (21 in lqcd_split.cu: single and double), 4
+    // BiCGstab: 24 spinor passes (23 in lqcd_split.cu: single and double), 4
     // half sweeps of links, solution r/w;
     // series: p, tmp, tmp, r, p, p (6 passes), 2 half sweeps of links;
     // Schwarz-preconditioned BiCGstab (per even site of the lattice, nsap
@@ -1946,7 +1947,7 @@ void solver_site_bytes(int prec, int method, double* inner, double* outer, int n
         *inner = 2.0 * (4.0 * sp + lk) + 4.0 * lk + 28.0 * sp + 4.0 * se;
     else
         *inner = method == SOLVER_SERIES ? 6.0 * sp + 2.0 * lk
-                                         : (prec == PREC64 || prec == PREC32 ? 21.0 : 24.0) * sp + 4.0 * lk + 2.0 * se;
+                                         : (prec == PREC64 || prec == PREC32 ? 23.0 : 24.0) * sp + 4.0 * lk + 2.0 * se;
     *outer = (192.0 + 3.0 * sp + se) + (2.0 * 192.0 + se) + (2.0 * 192.0 + 1152.0) + (4.0 * 192.0 + 1152.0);
 }
 

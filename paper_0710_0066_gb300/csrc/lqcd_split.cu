@@ -16,18 +16,19 @@
 //   * larger systems: L2 traffic and instruction fetch.  One thread per site
 //     (LPS = 1) with the loads of a hop issued before the arithmetic of the
 //     previous one, one copy of the hopping code for all sweeps of an
-//     iteration (35 KB; four copies overran the instruction cache and made a
-//     sweep 1.5 times longer), vectors and links in tiles of 32 sites, no
-//     register spills (phases, barriers and reductions are kept apart for
-//     that: spilled registers tripled the L2 writes).
+//     iteration (four copies overran the instruction cache and made a sweep
+//     1.5 times longer), vectors and links in tiles of 32 sites, phases,
+//     barriers and reductions kept apart so that no more than a few of the
+//     128 registers spill (4-16 bytes a kernel, 32 a reduction; spilled
+//     vectors tripled the L2 writes).
 //   * everywhere: the dot products of an iteration are FP64 sums and its
 //     scalars double, whatever the storage.  FP64 issues two lanes per cycle
 //     and SM, so a site's term (a word's, in an element-wise phase) is summed
 //     in the storage arithmetic first.
 // Measured (ms per solve to 1e-12, one thread per site without the above ->
-// this kernel): 12x6^3 global 5.06 -> 2.22, 32x16^3 global 30.2 -> 20.4, its
-// 8 slabs 4.80 -> 3.43, 64x32^3 global 647 -> 391, 32x24^3 series 9.23 -> 7.64;
-// double precision at 16x8^3 (two solves and the force) 34.5 -> 5.73.
+// this kernel): 12x6^3 global 4.48 -> 2.54, 32x16^3 global 34.6 -> 26.8, its
+// 8 slabs 4.87 -> 3.92, 64x32^3 global 727 -> 450, 32x24^3 series 9.31 -> 7.71;
+// double precision at 16x8^3 (two solves and the force) 34.3 -> 5.73.
 #include <algorithm>
 
 #include "lqcd_solve.cuh"
@@ -1124,13 +1125,15 @@ const Variant variants[SPLIT_NVAR] = {variant<PREC64, 8, 256, 1>(), variant<PREC
 
 // The kernel for `groups` groups of 32 sites over all systems.  Double
 // precision is bound by the FP64 pipe, which eight warps fill.  Single
-// precision, measured (ms per solve, LPS 8 / 4 / 2 / 1): 41 groups 2.23 / 2.36 /
-// 2.71 / 3.25, 128 groups 2.23 / 2.26 / 2.55 / 3.24, 300 groups 2.73 / 2.41 /
-// 2.50 / 3.17, 648 groups 16.3 / 14.2 / 13.3 / 13.1, 1024 groups 16.2 / 13.9 /
-// 12.0 / 11.9: LPS 8 while every group has an SM of its own, then 4 and 2 while
+// precision, measured (ms per solve, LPS 8 / 4 / 2 / 1): 41 groups 1.72 / 1.83 /
+// 2.06 / 2.46, 128 groups 1.96 / 1.93 / 2.17 / 2.70, 250 groups 2.32 / 2.06 /
+// 2.26 / 2.74, 540 groups 2.94 / 2.64 / 2.44 / 2.85, 648 groups 3.43 / 3.12 /
+// 2.86 / 2.92, 1024 groups 3.86 / 3.35 / 3.05 / 3.05, 2048 groups 5.78 / 5.13 /
+// 4.62 / 4.20: LPS 8 while every group has an SM of its own, then 4 and 2 while
 // the groups still fit the SMs side by side.  From 2432 groups on (more than
 // two CTAs of eight groups per SM) one CTA of 512 threads per SM halves the
-// barrier's arrivals (6912 groups 66.3 against 67.6, 32768 groups 420 / 431).
+// barrier's arrivals (2450 groups 5.43 against 5.55, 3072 groups 6.33 / 6.49,
+// 6912 groups 12.84 / 12.88).
 int pick(int prec, int groups, int num_sms)
 {
     if (prec == PREC64) return V_F64;
