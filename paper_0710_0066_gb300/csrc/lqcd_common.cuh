@@ -246,6 +246,23 @@ LQ_HD void accum_recon1(int mu, int sg, const cx<T>& w0, const cx<T>& w1, Spinor
     if (sg < 0) { acc.c[2][i] = acc.c[2][i] - l0; acc.c[3][i] = acc.c[3][i] - l1; }
     else        { acc.c[2][i] = acc.c[2][i] + l0; acc.c[3][i] = acc.c[3][i] + l1; }
 }
+// the same, acc set instead of added to
+template <class T>
+LQ_HD void set_recon1(int mu, int sg, const cx<T>& w0, const cx<T>& w1, Spinor<T>& acc, int i)
+{
+    acc.c[0][i] = w0;
+    acc.c[1][i] = w1;
+    switch (mu) {
+        case 0: acc.c[2][i] = -w0; acc.c[3][i] = -w1; break;
+        case 1: acc.c[2][i] = mul_i(w1); acc.c[3][i] = mul_i(w0); break;
+        case 2: acc.c[2][i] = w1; acc.c[3][i] = -w0; break;
+        default: acc.c[2][i] = mul_i(w0); acc.c[3][i] = mul_mi(w1); break;
+    }
+    if (sg < 0) {
+        acc.c[2][i] = -acc.c[2][i];
+        acc.c[3][i] = -acc.c[3][i];
+    }
+}
 
 template <class T>
 LQ_HD void project(int mu, int sg, const Spinor<T>& p, HalfSp<T>& h)

@@ -329,13 +329,24 @@ __device__ __forceinline__ cx<T> cmul1(cx<T> a, cx<T> b)
 
 // adds hop H: the neighbour is projected, and the link applied and the result
 // accumulated colour by colour (row by row, column by column for U^dag), so
-// that besides acc only the half spinor and rows 0-1 of the link are live
-template <int P, int H>
+// that besides acc only the half spinor and rows 0-1 of the link are live.
+// FIRST: acc is set instead (with a warp per hop, adding to zero would be 192
+// of a site's 1200 additions and multiply-adds: a series at 64x32^3 in double,
+// bound by their number, took 131 instead of 123 ms)
+template <int P, int H, bool FIRST>
 __device__ __forceinline__ void hop_add(const Raw<P>& R, Spinor<typename Real<P>::T>& acc)
 {
     typedef typename Real<P>::T T;
     constexpr int MU = 3 - H / 2, DAG = H & 1, sg = DAG ? +1 : -1;
-    if (MU == 0 && !R.use) return;
+    if (MU == 0 && !R.use) {
+        if (FIRST) {
+#pragma unroll
+            for (int s = 0; s < 4; ++s)
+#pragma unroll
+                for (int c = 0; c < 3; ++c) acc.c[s][c] = mk(T(0), T(0));
+        }
+        return;
+    }
     HalfSp<T> h;
     {
         Spinor<T> s;
@@ -358,13 +369,14 @@ __device__ __forceinline__ void hop_add(const Raw<P>& R, Spinor<typename Real<P>
             w0 = -w0;
             w1 = -w1;
         }
-        accum_recon1(MU, sg, w0, w1, acc, c);
+        if (FIRST) set_recon1(MU, sg, w0, w1, acc, c);
+        else accum_recon1(MU, sg, w0, w1, acc, c);
     }
 }
 
 // hops H, H + STEP, .. (N of them): the loads of a hop are issued before the
 // arithmetic of the one before it
-template <int P, int H, int STEP, int N>
+template <int P, int H, int STEP, int N, bool FIRST = true>
 struct Hops {
     static __device__ __forceinline__ void run(const Geo& g, int mode, int pout, int i, const int x[4], int lex,
                                                const typename Word<P>::W* in, const GaugeF& U, Raw<P>& R,
@@ -373,10 +385,10 @@ struct Hops {
         if constexpr (N > 1) {
             Raw<P> Q;
             hop_fetch<P, H + STEP>(g, mode, pout, i, x, lex, in, U, Q);
-            hop_add<P, H>(R, acc);
-            Hops<P, H + STEP, STEP, N - 1>::run(g, mode, pout, i, x, lex, in, U, Q, acc);
+            hop_add<P, H, FIRST>(R, acc);
+            Hops<P, H + STEP, STEP, N - 1, false>::run(g, mode, pout, i, x, lex, in, U, Q, acc);
         } else {
-            hop_add<P, H>(R, acc);
+            hop_add<P, H, FIRST>(R, acc);
         }
     }
     static __device__ __forceinline__ void start(const Geo& g, int mode, int pout, int i, const int x[4], int lex,
@@ -394,11 +406,6 @@ template <int P, int LPS>
 __device__ __forceinline__ void hop_part(const Geo& g, int mode, int pout, int i, int d, const typename Word<P>::W* in,
                                          const GaugeF& U, Spinor<typename Real<P>::T>& acc)
 {
-    typedef typename Real<P>::T T;
-#pragma unroll
-    for (int s = 0; s < 4; ++s)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) acc.c[s][c] = mk(T(0), T(0));
     int x[4];
     eo_coords(g, pout, i, x);
     const int lex = lex_of(g, x);
@@ -1119,13 +1126,16 @@ constexpr Variant variant()
 }
 
 enum { V_F64 = 0, V_8, V_4, V_2, V_1, V_1W };
-const Variant variants[SPLIT_NVAR] = {variant<PREC64, 8, 256, 1>(), variant<PREC32, 8, 256, 2>(),
+const Variant variants[SPLIT_NVAR] = {variant<PREC64, 8, 256, 2>(), variant<PREC32, 8, 256, 2>(),
                                       variant<PREC32, 4, 256, 2>(), variant<PREC32, 2, 256, 2>(),
                                       variant<PREC32, 1, 256, 2>(), variant<PREC32, 1, 512, 1>()};
 
 // The kernel for `groups` groups of 32 sites over all systems.  Double
-// precision is bound by the FP64 pipe, which eight warps fill.  Single
-// precision, measured (ms per solve, LPS 8 / 4 / 2 / 1): 41 groups 1.72 / 1.83 /
+// precision is bound by the FP64 pipe: eight warps a group, two CTAs per SM so
+// that one computes while the other's loads or barriers are under way (at
+// 128 registers a thread; one CTA of 255 registers: 64x32^3 global 206 ms
+// instead of 171, its series 123 / 99.5, 32x16^3 global 13.7 / 12.6; one thread
+// per site: 198, 112, 15.5).  Single precision, measured (ms per solve, LPS 8 / 4 / 2 / 1): 41 groups 1.72 / 1.83 /
 // 2.06 / 2.46, 128 groups 1.96 / 1.93 / 2.17 / 2.70, 250 groups 2.32 / 2.06 /
 // 2.26 / 2.74, 540 groups 2.94 / 2.64 / 2.44 / 2.85, 648 groups 3.43 / 3.12 /
 // 2.86 / 2.92, 1024 groups 3.86 / 3.35 / 3.05 / 3.05, 2048 groups 5.78 / 5.13 /
@@ -1195,8 +1205,23 @@ SplitPlan split_plan(SolveArgs& A, int prec, int method, int spt, int num_sms, c
     const Variant& v = variants[k];
     const int SG = v.bs / 32 / v.lps;  // groups a CTA holds side by side
     const int want = spt <= 0 ? G : (G + SG * spt - 1) / (SG * spt);
-    A.cps = std::max(1, std::min(occ[k][m] * num_sms / A.ngrp, want));
-    const int gpc = (G + A.cps - 1) / A.cps;
+    auto groups_per_cta = [&](int per_sm) {
+        A.cps = std::max(1, std::min(per_sm * num_sms / A.ngrp, want));
+        return (G + A.cps - 1) / A.cps;
+    };
+    // Double precision: the FP64 pipe of the SM with the most groups sets the
+    // time, so one CTA per SM where two would leave that SM with over a tenth
+    // more groups (420 groups by two 3.61 ms, by one 3.11; 1024: 6.94 / 6.51,
+    // 2048, where both give 14: 12.6 / 13.7)
+    int per_sm = occ[k][m];
+    if (prec == PREC64 && per_sm > 1) {
+        auto most = [&](int n) {
+            const int gpc = groups_per_cta(n), ctas = (G + gpc - 1) / gpc * A.ngrp;
+            return (ctas + num_sms - 1) / num_sms * gpc;
+        };
+        if (11 * most(1) < 10 * most(per_sm)) per_sm = 1;
+    }
+    const int gpc = groups_per_cta(per_sm);
     A.cps = (G + gpc - 1) / gpc;
     A.chunk = gpc * 32;
     // tiles of 16 groups where the CTAs make several passes (64x32^3: 420
