@@ -178,12 +178,13 @@ __device__ __forceinline__ void hop_body(Geo g, int mode, int dag, int pout, int
     int i = on ? t : nsites - 1;
     bool mine = true;
     if (colour >= 0) {
-        if (ABI) {  // every site, zeros on the other colour's slabs
-            mine = ((i / g.Sh) & 1) == colour;
-        } else {
-            const int k = t / g.Sh;
-            i = (colour + 2 * k) * g.Sh + (t - k * g.Sh);
-        }
+        // with ABI every site: first the colour's, then zeros on the other
+        // slabs (the sites in their own order would give one SM two blocks of
+        // work and the next none: 16^4 in double 0.168 ms instead of 0.131)
+        const int half = (g.nb / 2) * g.Sh;
+        mine = !ABI || i < half;
+        const int u = mine ? i : i - half, k = u / g.Sh;
+        i = ((mine ? colour : 1 - colour) + 2 * k) * g.Sh + (u - k * g.Sh);
     }
     Spinor<T> acc;
     if (mine) {
