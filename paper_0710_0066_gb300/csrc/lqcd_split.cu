@@ -26,9 +26,9 @@
 //     and SM, so a site's term (a word's, in an element-wise phase) is summed
 //     in the storage arithmetic first.
 // Measured (ms per solve to 1e-12, one thread per site without the above ->
-// this kernel): 12x6^3 global 4.48 -> 2.54, 32x16^3 global 34.6 -> 26.8, its
-// 8 slabs 4.87 -> 3.92, 64x32^3 global 727 -> 450, 32x24^3 series 9.31 -> 7.71;
-// double precision at 16x8^3 (two solves and the force) 34.3 -> 5.73.
+// this kernel): 12x6^3 global 4.65 -> 2.61, 32x16^3 global 30.7 -> 24.0, its
+// 8 slabs 4.77 -> 3.83, 64x32^3 global 579 -> 358, 32x24^3 series 9.37 -> 7.70;
+// double precision at 16x8^3 (two solves and the force) 34.9 -> 5.70.
 #include <algorithm>
 
 #include "lqcd_solve.cuh"
@@ -1135,15 +1135,15 @@ const Variant variants[SPLIT_NVAR] = {variant<PREC64, 8, 256, 2>(), variant<PREC
 // that one computes while the other's loads or barriers are under way (at
 // 128 registers a thread; one CTA of 255 registers: 64x32^3 global 206 ms
 // instead of 171, its series 123 / 99.5, 32x16^3 global 13.7 / 12.6; one thread
-// per site: 198, 112, 15.5).  Single precision, measured (ms per solve, LPS 8 / 4 / 2 / 1): 41 groups 1.72 / 1.83 /
-// 2.06 / 2.46, 128 groups 1.96 / 1.93 / 2.17 / 2.70, 250 groups 2.32 / 2.06 /
-// 2.26 / 2.74, 540 groups 2.94 / 2.64 / 2.44 / 2.85, 648 groups 3.43 / 3.12 /
-// 2.86 / 2.92, 1024 groups 3.86 / 3.35 / 3.05 / 3.05, 2048 groups 5.78 / 5.13 /
-// 4.62 / 4.20: LPS 8 while every group has an SM of its own, then 4 and 2 while
-// the groups still fit the SMs side by side.  From 2432 groups on (more than
-// two CTAs of eight groups per SM) one CTA of 512 threads per SM halves the
-// barrier's arrivals (2450 groups 5.43 against 5.55, 3072 groups 6.33 / 6.49,
-// 6912 groups 12.84 / 12.88).
+// per site: 198, 112, 15.5).  Single precision, measured (ms per solve, LPS 8 / 4 / 2 / 1):
+// 41 groups 1.72 / 1.84 / 2.09 / 2.42, 128 groups 1.97 / 1.96 / 2.20 / 2.77, 250
+// groups 2.39 / 2.07 / 2.26 / 2.81, 540 groups 2.88 / 2.60 / 2.43 / 2.79, 648
+// groups 3.39 / 3.03 / 2.94 / 2.91, 1024 groups 3.69 / 3.33 / 2.97 / 2.98, 2048
+// groups 5.83 / 5.01 / 4.53 / 4.22: LPS 8 while every group has an SM of its own,
+// then 4 and 2 while the groups still fit the SMs side by side.  From 2432
+// groups on (more than two CTAs of eight groups per SM) one CTA of 512 threads
+// per SM halves the barrier's arrivals (2450 groups 5.64 against 5.74, 3072
+// groups 6.15 / 6.37, 6912 groups 13.44 / 13.49).
 int pick(int prec, int groups, int num_sms)
 {
     if (prec == PREC64) return V_F64;
