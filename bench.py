@@ -82,9 +82,9 @@ PEAKS = os.path.join(ROOT, "MEASURED_PEAKS.json")
 # precision, valid only for the solver source that was captured (bench.py
 # reports null once the source differs)
 SOLVER_SOURCES = ("lqcd_split.cu", "lqcd_solve.cuh", "lqcd_common.cuh", "lqcd_df.cuh")  # the sources k_split is built from
-SOLVER_TRAFFIC = dict(src_sha256="d361f8bf57e40fdc75a5514e4db0ebe94ea8c46190e0eda92521a7be04447471",
-                      block_series=(346.314e6 + 147.963e6), block=(426.858e6 + 442.421e6),
-                      glob=(515.311e6 + 604.961e6))
+SOLVER_TRAFFIC = dict(src_sha256="e767fb577af8c16321f0844dd231ae682b37cc22b8096f0784baba48f282bc09",
+                      block_series=(336.252e6 + 145.905e6), block=(440.540e6 + 547.191e6),
+                      glob=(536.571e6 + 768.481e6))
 
 
 def solver_traffic():
